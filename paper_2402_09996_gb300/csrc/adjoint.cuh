@@ -73,7 +73,7 @@ __device__ __forceinline__ void stage_eval(const MatDev<T>& M, const T* e0, cons
   V.Rb_s = M.Q_s * (M.h_off * (T(12) - V.Es) + dq);
   V.Rb_t = M.Q_b * (M.h_off * (T(4) - V.Et) + dq);
   RootCoef<T> qs, qt;
-  if constexpr (NP != 0 && SOLVE) {
+  if constexpr (NP != 0 && NP != kDirect && SOLVE) {
     qs = root_coef<T>(T(1), M.K, M.n, M.inv_n, M.lg_K, M.eta, M.lg_eta, T(0));
     qt = root_coef<T>(V.Ptw, M.Kt, M.nt, M.inv_nt, M.lg_Kt, M.eta, M.lg_eta, V.lg_Ptw);
   }
@@ -552,8 +552,7 @@ __global__ void k_material_point_vjp(const MatDev<T> M, long long nvox, const T*
                                      const T* __restrict__ root_tab) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* tab = reinterpret_cast<T*>(smem_raw);
-  if (NP != 0)
-    for (int k = threadIdx.x; k < kRootTabs; k += blockDim.x) tab[k] = root_tab[k];
+  stage_tables<T>(tab, root_tab, table_len<T, NP>(M));
   __syncthreads();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nvox) return;
@@ -597,8 +596,7 @@ __global__ void k_adj_tangent(const MatDev<T> M, long long nvox, const T* __rest
                               const T* __restrict__ root_tab) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* tab = reinterpret_cast<T*>(smem_raw);
-  if (NP != 0)
-    for (int k = threadIdx.x; k < kRootTabs; k += blockDim.x) tab[k] = root_tab[k];
+  stage_tables<T>(tab, root_tab, table_len<T, NP>(M));
   __syncthreads();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nvox) return;

@@ -399,11 +399,22 @@ void release(rve_s* h) {
   h->st_host = nullptr;
 }
 
-// The x pass stages the two rate-root tables (kRootTabs values) in shared memory after
-// its FFT buffers.
+// Rate-solve variant of a material, whether its slip and twin laws need a table each, and the
+// number of values of its tables (rate_table.cuh; kRootTabs for the Newton variants).
+template <typename T>
+int variant_of(const rve_material& m) { return rate_variant<T>(m.eta, m.K, m.n, m.Kt, m.nt); }
+bool two_laws(const rve_material& m) { return m.K != m.Kt || m.n != m.nt; }
+template <typename T>
+size_t tables_of(const rve_material& m) {
+  const int np = variant_of<T>(m);
+  return np == kDirect ? (size_t)rate_tab_len<T>(two_laws(m)) : (np == 0 ? 0 : (size_t)kRootTabs);
+}
+
+// The x pass stages the rate tables in shared memory before its FFT buffers.
 size_t xsmem_total(const rve_s* h) {
-  const size_t elem = h->opt.precision == RVE_FP64 ? sizeof(double) : sizeof(float);
-  return h->xsmem + (size_t)kRootTabs * elem;
+  const rve_material& m = h->mat;
+  if (h->opt.precision == RVE_FP64) return h->xsmem + tables_of<double>(m) * sizeof(double);
+  return h->xsmem + tables_of<float>(m) * sizeof(float);
 }
 
 template <typename T>
@@ -432,6 +443,18 @@ MatDev<T> make_mat(const rve_s* h) {
   const double sc = 1.0 / std::sqrt(6.0);
   M.C11s = (T)(m.C11 * sc); M.C12s = (T)(m.C12 * sc); M.C13s = (T)(m.C13 * sc); M.C33s = (T)(m.C33 * sc);
   M.C44s2 = (T)(2.0 * m.C44 * sc); M.C66s2 = (T)(2.0 * m.C66 * sc);
+  M.ls = M.lt = RateLaw<T>{};
+  M.inv_ntm1 = (T)0;
+  M.rate_len = 0;
+  if (variant_of<T>(m) == kDirect) {
+    RateGrid g0, g1;
+    rate_law_fit_t<T>(m.K, m.n, m.eta, &g0);
+    rate_law_fit_t<T>(m.Kt, m.nt, m.eta, &g1);
+    M.ls = rate_law<T>(g0, 0);
+    M.lt = rate_law<T>(g1, two_laws(m) ? RateFmt<T>::kLen : 0);
+    M.inv_ntm1 = (T)(1.0 / (m.nt - 1.0));
+    M.rate_len = rate_tab_len<T>(two_laws(m));
+  }
   return M;
 }
 
@@ -647,13 +670,26 @@ std::vector<T> root_tables(const rve_material& m) {
   return std::vector<T>(d.begin(), d.end());
 }
 
+// The material's rate tables on the device: direct tables are built by a kernel, the Newton
+// variants' start tables on the host.
 template <typename T>
 rve_status upload_root_tab(rve_s* h) {
-  const std::vector<T> t = root_tables<T>(h->mat);
+  const rve_material& m = h->mat;
+  const int np = variant_of<T>(m);
   if (!h->root_tab) {
-    rve_status s = dalloc(h, &h->root_tab, (size_t)kRootTabs * sizeof(T));
+    // room for any material of the handle
+    rve_status s = dalloc(h, &h->root_tab, std::max((size_t)kRootTabs, (size_t)rate_tab_len<T>(true)) * sizeof(T));
     if (s) return s;
   }
+  if (np == 0) return RVE_OK;
+  if (np == kDirect) {
+    RateGrid g0, g1;
+    rate_law_fit_t<T>(m.K, m.n, m.eta, &g0);
+    rate_law_fit_t<T>(m.Kt, m.nt, m.eta, &g1);
+    RVE_CUDA(h, launch_rate_table<T>((T*)h->root_tab, two_laws(m), g0, g1, m.K, m.n, m.Kt, m.nt, m.eta, h->stream));
+    return RVE_OK;
+  }
+  const std::vector<T> t = root_tables<T>(m);
   RVE_CUDA(h, cudaMemcpyAsync(h->root_tab, t.data(), t.size() * sizeof(T), cudaMemcpyHostToDevice, h->stream));
   RVE_CUDA(h, cudaStreamSynchronize(h->stream));
   return RVE_OK;
@@ -813,7 +849,8 @@ int max_iter_of(const rve_s* h) { return h->opt.max_iter > 0 ? h->opt.max_iter :
 
 int np_of(const rve_s* h) {
   const rve_material& m = h->mat;
-  return h->lin_mode ? kLinearLaw : rate_variant(m.eta, m.K, m.Kt, is_small_int(m.n), is_small_int(m.nt));
+  if (h->lin_mode) return kLinearLaw;
+  return h->opt.precision == RVE_FP64 ? variant_of<double>(m) : variant_of<float>(m);
 }
 
 // One fixed-point iteration (x pass, forward y, z + Green, inverse y) on stream s:
@@ -1569,8 +1606,7 @@ rve_status adjoint_increment(rve_s* h, const double* eps_prev, const double* eps
   T* A = (T*)h->adj;
   auto at = [&](int slot) { return A + (size_t)slot * N; };
   const MatDev<T> M = make_mat<T>(h);
-  const rve_material& m = h->mat;
-  const int np = rate_variant(m.eta, m.K, m.Kt, is_small_int(m.n), is_small_int(m.nt));
+  const int np = variant_of<T>(h->mat);
   const int nsub = h->opt.n_sub > 0 ? h->opt.n_sub : default_nsub(dt_n);
   if (nsub > kMaxSubVjp) return fail(h, RVE_ERR_UNSUPPORTED, "adjoint: more than 16 RK4 substeps per increment");
   const T dt = (T)dt_n;
@@ -2221,7 +2257,7 @@ rve_status rve_material_point(int precision, const rve_material* mat, long long 
   if (precision != RVE_FP64 && precision != RVE_FP32) return fail(nullptr, RVE_ERR_INVALID_ARG, "bad precision");
   cudaStream_t st = stream ? (cudaStream_t)stream : cudaStreamPerThread;
   tmp.stream = st;
-  const int np = rate_variant(mat->eta, mat->K, mat->Kt, is_small_int(mat->n), is_small_int(mat->nt));
+  const int np = precision == RVE_FP64 ? variant_of<double>(*mat) : variant_of<float>(*mat);
   s = precision == RVE_FP64 ? upload_root_tab<double>(&tmp) : upload_root_tab<float>(&tmp);
   if (s) {
     release(&tmp);
@@ -2258,7 +2294,7 @@ rve_status rve_material_point_vjp(int precision, const rve_material* mat, long l
   if (precision != RVE_FP64 && precision != RVE_FP32) return fail(nullptr, RVE_ERR_INVALID_ARG, "bad precision");
   cudaStream_t st = stream ? (cudaStream_t)stream : cudaStreamPerThread;
   tmp.stream = st;
-  const int np = rate_variant(mat->eta, mat->K, mat->Kt, is_small_int(mat->n), is_small_int(mat->nt));
+  const int np = precision == RVE_FP64 ? variant_of<double>(*mat) : variant_of<float>(*mat);
   s = precision == RVE_FP64 ? upload_root_tab<double>(&tmp) : upload_root_tab<float>(&tmp);
   if (s) {
     release(&tmp);

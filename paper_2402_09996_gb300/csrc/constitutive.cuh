@@ -17,13 +17,17 @@
 // increment (Sec. 3, "explicit ... Runge-Kutta 4th order").
 //
 // Template parameter NP selects how the regularised rates are solved:
-//   NP > 0   eta > 0 and n = nt = NP (compile-time power): table start, branch-free;
-//   NP = -1  eta > 0, any real n, nt >= 1 (powers as 2^(p log2 z)): table start, branch-free;
-//   NP = 0   anything else (eta = 0 or non-integer exponents): generic per-system solve.
+//   NP = kDirect  eta > 0 and both laws tabulated directly (rate_table.cuh): no solve;
+//   NP = 10       double, eta > 0 and n = nt = 10 (compile-time power): table start,
+//                 branch-free;
+//   NP = -1       eta > 0, any real n, nt >= 1 (powers as 2^(p log2 z)): table start,
+//                 branch-free;
+//   NP = 0        eta = 0, and arguments outside the direct tables: generic per-system solve.
 #pragma once
 
 #include <type_traits>
 
+#include "rate_table.cuh"
 #include "rve_common.cuh"
 
 namespace rve {
@@ -294,7 +298,6 @@ template <> struct TabNewton<double> { static constexpr int value = 3; };
 template <typename T>
 struct RootCoef {
   T Pout, c, cn, Kn, Kn_n, a1, b1, a2, b2, nm1;
-  T lo;  // argument floor of the packed float solves with a compile-time power (root_floor)
 };
 
 template <typename T>
@@ -311,20 +314,7 @@ __device__ __forceinline__ RootCoef<T> root_coef(T P, T Kn, T n, T inv_n, T lg_K
   q.a2 = (inv_n - T(1)) * T(kRootPerUnit);
   q.b2 = (lg_Kn + q.b1 + T(kRootSpan)) * T(kRootPerUnit) - T(0.5);
   q.nm1 = n - T(1);
-  q.lo = T(0);
   return q;
-}
-
-// The argument whose table coordinate is kRootIv - 1.25, i.e. 3/4 of an interval inside the
-// table's upper end (a2 < 0 for n > 1: larger arguments map to smaller coordinates).  The
-// packed solves with a compile-time power floor their arguments here, so that their table
-// index needs a lower clamp only.  At this argument the root sits on the Norton asymptote
-// 2^16 below the kink, and the rate (a/eta) u*^n is below 2^-160 whenever eta >= K (the
-// host selects this variant only then), so it rounds to exactly 0 in float: every argument
-// at or below the floor -- inactive systems (a <= 0), NaN, and the positive arguments whose
-// exact rate underflows -- returns the masked form's value 0.
-__device__ __forceinline__ float root_floor(const RootCoef<float>& q) {
-  return fast_exp2<float>(__fdividef(float(kRootIv) - 1.25f - q.b2, q.a2));
 }
 
 // z^(n-1) for the table-started Newton steps (z > 0): a compile-time product for NP > 0,
@@ -413,29 +403,15 @@ __device__ __forceinline__ T reg_rate_slip(T a, const RootCoef<T>& q, int n_int,
 // logarithms, exponentials and reciprocals stay per lane.
 __device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
 
-template <int NP>
-__device__ __forceinline__ float2 root_zn1_2(float2 z, const RootCoef<float>& q, int n_int) {
-  if constexpr (NP > 0) {
-    // z^(NP-1) by the binary powering of cpow<NP - 1>, both lanes at once
-    float2 r = z;
-    constexpr int e = NP - 1;
-    if constexpr (e == 9) {
-      const float2 h2 = __fmul2_rn(z, z), h4 = __fmul2_rn(h2, h2), h8 = __fmul2_rn(h4, h4);
-      r = __fmul2_rn(z, h8);
-    } else {
-      r = make_float2(cpow<NP - 1, float>(z.x), cpow<NP - 1, float>(z.y));
-    }
-    return r;
-  } else {
-    const float2 l = __fmul2_rn(f2(q.nm1), make_float2(fast_log2<float>(z.x), fast_log2<float>(z.y)));
-    return make_float2(fast_exp2<float>(l.x), fast_exp2<float>(l.y));
-  }
+__device__ __forceinline__ float2 root_zn1_2(float2 z, const RootCoef<float>& q) {
+  const float2 l = __fmul2_rn(f2(q.nm1), make_float2(fast_log2<float>(z.x), fast_log2<float>(z.y)));
+  return make_float2(fast_exp2<float>(l.x), fast_exp2<float>(l.y));
 }
 
 // UNIT_P: the slip systems' prefactor P = 1 (no final scaling).
-template <int NP, bool UNIT_P = false>
-__device__ __forceinline__ float2 root_newton2(float2 z, float2 aa, const RootCoef<float>& q, int n_int) {
-  const float2 zn1 = root_zn1_2<NP>(z, q, n_int);
+template <bool UNIT_P = false>
+__device__ __forceinline__ float2 root_newton2(float2 z, float2 aa, const RootCoef<float>& q) {
+  const float2 zn1 = root_zn1_2(z, q);
   const float2 phi = __ffma2_rn(z, __ffma2_rn(f2(q.c), zn1, f2(q.Kn)), make_float2(-aa.x, -aa.y));
   const float2 den = __ffma2_rn(f2(q.c), zn1, f2(q.Kn_n));
   const float2 r = make_float2(fast_rcp<float>(den.x), fast_rcp<float>(den.y));
@@ -444,65 +420,34 @@ __device__ __forceinline__ float2 root_newton2(float2 z, float2 aa, const RootCo
   else return __fmul2_rn(f2(q.Pout), __fmul2_rn(zn1, w));
 }
 
-// With a compile-time power (NP = n = nt = 10) an inactive system (a <= 0, or NaN) is solved
-// at the floor q.lo (root_floor) instead of being masked: its rate rounds to exactly 0 --
-// the masked form's value -- while one min replaces a compare and two selects per system,
-// and the floor bounds the table coordinate from above.  A real exponent near 1 would not
-// underflow, so NP = -1 keeps the mask.
-template <int NP>
-__device__ __forceinline__ float2 rate_arg2(float2 a, float lo) {
-  if constexpr (NP > 0) return make_float2(fmaxf(a.x, lo), fmaxf(a.y, lo));
-  else return make_float2(a.x > 0.f ? a.x : 1.f, a.y > 0.f ? a.y : 1.f);
-}
-
-// Table entries at the coordinates t of a pair.  NP > 0: t <= kRootIv - 1.25 (floored
-// arguments), so only the lower clamp remains; it is taken in float on t rounded at the
-// 1.5 * 2^23 binade (any t, -inf included, gives an index in [0, kRootIv - 1]), and the
-// binade's offset folds into the table address.
-template <int NP>
-__device__ __forceinline__ void tab_pair(float2 t, const float* tab, float2& ab0, float2& ab1) {
-  const float2* tb = reinterpret_cast<const float2*>(tab);
-  if constexpr (NP > 0) {
-    const float2 m = __fadd2_rn(t, f2(12582912.0f));
-    ab0 = tb[__float_as_int(fmaxf(m.x, 12582912.0f)) - 0x4B400000];
-    ab1 = tb[__float_as_int(fmaxf(m.y, 12582912.0f)) - 0x4B400000];
-  } else {
-    ab0 = tb[root_interval<float>(t.x)];
-    ab1 = tb[root_interval<float>(t.y)];
-  }
-}
-template <int NP>
+// Inactive systems (a <= 0, or NaN) are solved at a dummy argument and masked.
+__device__ __forceinline__ float2 rate_arg2(float2 a) { return make_float2(a.x > 0.f ? a.x : 1.f, a.y > 0.f ? a.y : 1.f); }
 __device__ __forceinline__ float2 rate_out2(float2 a, float2 rho) {
-  if constexpr (NP > 0) return rho;
-  else return make_float2(a.x > 0.f ? rho.x : 0.f, a.y > 0.f ? rho.y : 0.f);
+  return make_float2(a.x > 0.f ? rho.x : 0.f, a.y > 0.f ? rho.y : 0.f);
 }
 
-template <int NP>
-__device__ __forceinline__ float2 reg_rate_slip2(float2 a, const RootCoef<float>& q, int n_int, const float* tab) {
-  const float2 aa = rate_arg2<NP>(a, q.lo);
+__device__ __forceinline__ float2 reg_rate_slip2(float2 a, const RootCoef<float>& q, const float* tab) {
+  const float2* tb = reinterpret_cast<const float2*>(tab);
+  const float2 aa = rate_arg2(a);
   const float2 la = make_float2(fast_log2<float>(aa.x), fast_log2<float>(aa.y));
   const float2 t = __ffma2_rn(la, f2(q.a2), f2(q.b2));
-  float2 ab0, ab1;
-  tab_pair<NP>(t, tab, ab0, ab1);
+  const float2 ab0 = tb[root_interval<float>(t.x)], ab1 = tb[root_interval<float>(t.y)];
   // one FMA per lane: the two systems' table entries are not an operand pair
   const float2 ex = make_float2(fmaf(ab0.y, la.x, ab0.x), fmaf(ab1.y, la.y, ab1.x));
   const float2 z = make_float2(fast_exp2<float>(ex.x), fast_exp2<float>(ex.y));
-  const float2 rho = root_newton2<NP, true>(z, aa, q, n_int);
-  return rate_out2<NP>(a, rho);
+  return rate_out2(a, root_newton2<true>(z, aa, q));
 }
 
-template <int NP>
-__device__ __forceinline__ float2 reg_rate_tab2(float2 a, const RootCoef<float>& q, int n_int, const float* tab) {
-  const float2 aa = rate_arg2<NP>(a, q.lo);
+__device__ __forceinline__ float2 reg_rate_tab2(float2 a, const RootCoef<float>& q, const float* tab) {
+  const float2* tb = reinterpret_cast<const float2*>(tab);
+  const float2 aa = rate_arg2(a);
   const float2 la = make_float2(fast_log2<float>(aa.x), fast_log2<float>(aa.y));
   const float2 lzB = __ffma2_rn(la, f2(q.a1), f2(q.b1));
   const float2 t = __ffma2_rn(la, f2(q.a2), f2(q.b2));
-  float2 ab0, ab1;
-  tab_pair<NP>(t, tab, ab0, ab1);
+  const float2 ab0 = tb[root_interval<float>(t.x)], ab1 = tb[root_interval<float>(t.y)];
   const float2 ex = __fadd2_rn(lzB, make_float2(fmaf(ab0.y, t.x, ab0.x), fmaf(ab1.y, t.y, ab1.x)));
   const float2 z = make_float2(fast_exp2<float>(ex.x), fast_exp2<float>(ex.y));
-  const float2 rho = root_newton2<NP>(z, aa, q, n_int);
-  return rate_out2<NP>(a, rho);
+  return rate_out2(a, root_newton2(z, aa, q));
 }
 
 // Generic solve (any eta >= 0 and exponent n >= 1): per-system branch, a smooth-minimum
@@ -536,11 +481,34 @@ __device__ __forceinline__ T reg_rate(T a, T P, T Kn, T n, int n_int, T inv_n, T
 }
 
 // ---------------------------------------------------------------- RK4 stage ----------
-// One regularised-rate solve: table start for NP != 0, generic otherwise.
+// The generic solve out of line, for arguments outside a direct table.
+template <typename T>
+__device__ __noinline__ T rate_generic(T a, T P, T Kn, T n, int n_int, T inv_n, T m, T lg_Kn, T eta, T lg_eta,
+                                       T lg_P) {
+  return reg_rate<T>(a, P, Kn, n, n_int, inv_n, m, lg_Kn, eta, lg_eta, lg_P);
+}
+
+// The twins' argument scale s = P^(1/(nt-1)) and its inverse for the direct table (both 0 for
+// P = 0: the rate is then 0).
+template <typename T>
+__device__ __forceinline__ void twin_scale(const MatDev<T>& M, T P, T lg_P, T* s, T* inv_s) {
+  const T l = lg_P * M.inv_ntm1;
+  *s = P > T(0) ? fast_exp2<T>(l) : T(0);
+  *inv_s = P > T(0) ? fast_exp2<T>(-l) : T(0);
+}
+
+// One regularised-rate solve: the direct table, a table start, or generic.
 template <typename T, int NP>
 __device__ __forceinline__ T stage_rate(const MatDev<T>& M, const RootCoef<T>& q, T a, T P, bool twin, T lg_P,
                                         const T* tab) {
-  if constexpr (NP != 0) {
+  if constexpr (NP == kDirect) {
+    T s = T(1), is = T(1);
+    if (twin) twin_scale<T>(M, P, lg_P, &s, &is);
+    const T rho = rate_direct(a * s, twin ? M.lt : M.ls, tab + (twin ? M.lt.off : M.ls.off)) * is;
+    if (rho == rho) return rho;
+    return twin ? rate_generic<T>(a, P, M.Kt, M.nt, M.nt_int, M.inv_nt, M.smt, M.lg_Kt, M.eta, M.lg_eta, lg_P)
+                : rate_generic<T>(a, P, M.K, M.n, M.n_int, M.inv_n, M.sm, M.lg_K, M.eta, M.lg_eta, lg_P);
+  } else if constexpr (NP != 0) {
     return twin ? reg_rate_tab<T, NP>(a, q, M.nt_int, tab + kRootTabLen) : reg_rate_slip<T, NP>(a, q, M.n_int, tab);
   } else {
     return twin ? reg_rate<T>(a, P, M.Kt, M.nt, M.nt_int, M.inv_nt, M.smt, M.lg_Kt, M.eta, M.lg_eta, lg_P)
@@ -550,7 +518,7 @@ __device__ __forceinline__ T stage_rate(const MatDev<T>& M, const RootCoef<T>& q
 
 // Packed two-lane solves: float with a table-started solve.
 template <typename T, int NP>
-constexpr bool kPackedSolve = std::is_same<T, float>::value && NP != 0;
+constexpr bool kPackedSolve = std::is_same<T, float>::value && NP < 0;
 
 // Two values of a pair of systems (or components).  Float: one packed two-lane FP32
 // instruction per operation; double: the scalar expressions.
@@ -669,13 +637,16 @@ __device__ __forceinline__ void rk_stage(const MatDev<T>& M, const T* e0, const 
   // the twins), as the host fills M.r0
   const T rb_sup = M.r0[0] + Rb_s, rb_ord = M.r0[2] + Rb_s, rb_tw = M.r0[12] + Rb_t;
   RootCoef<T> qs, qt;
-  if constexpr (NP != 0) {
+  if constexpr (NP != 0 && NP != kDirect) {
     qs = root_coef<T>(T(1), M.K, M.n, M.inv_n, M.lg_K, M.eta, M.lg_eta, T(0));
     qt = root_coef<T>(Ptw, M.Kt, M.nt, M.inv_nt, M.lg_Kt, M.eta, M.lg_eta, lg_Ptw);
-    if constexpr (kPackedSolve<T, NP> && NP > 0) {
-      qs.lo = root_floor(qs);
-      qt.lo = root_floor(qt);
-    }
+  }
+  T s_tw = T(0), is_tw = T(0);
+  const T *tab_s = tab, *tab_t = tab;
+  if constexpr (NP == kDirect) {
+    twin_scale<T>(M, Ptw, lg_Ptw, &s_tw, &is_tw);
+    tab_s = tab + M.ls.off;
+    tab_t = tab + M.lt.off;
   }
   // plane sums of the slip-scaled stress (plane_sum)
   T S[4][3];
@@ -697,8 +668,11 @@ __device__ __forceinline__ void rk_stage(const MatDev<T>& M, const T* e0, const 
     const T ak0 = fabs(tek0) - rr.x;
     const T ak1 = fabs(tek1) - rr.y;
     T rk2[2];
-    if constexpr (kPackedSolve<T, NP>) {
-      const float2 r = reg_rate_slip2<NP>(make_float2(ak0, ak1), qs, M.n_int, tab);
+    if constexpr (NP == kDirect) {
+      rk2[0] = rate_direct(ak0, M.ls, tab_s);
+      rk2[1] = rate_direct(ak1, M.ls, tab_s);
+    } else if constexpr (kPackedSolve<T, NP>) {
+      const float2 r = reg_rate_slip2(make_float2(ak0, ak1), qs, tab);
       rk2[0] = r.x;
       rk2[1] = r.y;
     } else {
@@ -738,8 +712,11 @@ __device__ __forceinline__ void rk_stage(const MatDev<T>& M, const T* e0, const 
     const T ak0 = kTw * plane_sum<T>(k, S[k - 12]) - rr.x;
     const T ak1 = kTw * plane_sum<T>(k + 1, S[k - 11]) - rr.y;
     T rk2[2];
-    if constexpr (kPackedSolve<T, NP>) {
-      const float2 r = reg_rate_tab2<NP>(make_float2(ak0, ak1), qt, M.nt_int, tab + kRootTabLen);
+    if constexpr (NP == kDirect) {
+      rk2[0] = rate_direct(ak0 * s_tw, M.lt, tab_t) * is_tw;
+      rk2[1] = rate_direct(ak1 * s_tw, M.lt, tab_t) * is_tw;
+    } else if constexpr (kPackedSolve<T, NP>) {
+      const float2 r = reg_rate_tab2(make_float2(ak0, ak1), qt, tab + kRootTabLen);
       rk2[0] = r.x;
       rk2[1] = r.y;
     } else {
@@ -917,6 +894,68 @@ __device__ __forceinline__ bool mc_voxel(const MatDev<T>& M, const T* R, const T
   hooke<T>(M, ee, sc);
   to_sample<T>(R, sc, sig);
   return flows;
+}
+
+// The whole update by the generic solve, out of line: voxels with an overstress beyond the
+// direct tables (their stress is NaN after mc_voxel<T, kDirect>), from the state at t_n.
+template <typename T>
+__device__ __noinline__ bool mc_voxel_generic(const MatDev<T>& M, const T* R, const T* eps_n, const T* eps,
+                                              MPState<T>& y, T dt, int nsub, T* sig) {
+  return mc_voxel<T, 0>(M, R, eps_n, eps, y, dt, nsub, sig, nullptr);
+}
+
+// Loads a voxel's state (component-major arrays of n voxels): eps_p, v, alpha.
+template <typename T>
+__device__ __forceinline__ void load_voxel(const T* ep, const T* v, const T* al, size_t n, size_t i, MPState<T>& y) {
+#pragma unroll
+  for (int c = 0; c < 6; ++c) y.ep[c] = ep[c * n + i];
+#pragma unroll
+  for (int c = 0; c < 16; ++c) y.v[c] = v[c * n + i];
+#pragma unroll
+  for (int c = 0; c < 12; ++c) y.al[c] = al[c * n + i];
+}
+
+// mc_voxel with the direct tables' out-of-range case: y holds the voxel's state at t_n, which
+// is also at (ep, v, al); the copies keep the arrays of the common path in registers.
+template <typename T, int NP>
+__device__ __forceinline__ bool mc_voxel_any(const MatDev<T>& M, const T* R, const T* eps_n, const T* eps,
+                                             MPState<T>& y, T dt, int nsub, T* sig, const T* tab, bool check,
+                                             const T* ep, const T* v, const T* al, size_t n, size_t i) {
+  const bool flows = mc_voxel<T, NP>(M, R, eps_n, eps, y, dt, nsub, sig, tab, check);
+  if constexpr (NP == kDirect && std::is_same<T, float>::value) {
+    if (sig[0] != sig[0]) {
+      T r2[9], a2[6], b2[6], s2[6];
+      MPState<T> y2;
+      load_voxel<T>(ep, v, al, n, i, y2);
+#pragma unroll
+      for (int c = 0; c < 9; ++c) r2[c] = R[c];
+#pragma unroll
+      for (int c = 0; c < 6; ++c) {
+        a2[c] = eps_n[c];
+        b2[c] = eps[c];
+      }
+      mc_voxel_generic<T>(M, r2, a2, b2, y2, dt, nsub, s2);
+      y = y2;
+#pragma unroll
+      for (int c = 0; c < 6; ++c) sig[c] = s2[c];
+    }
+  }
+  return flows;
+}
+
+// Copies the rate tables (a multiple of 16 bytes) to shared memory; no barrier.
+template <typename T>
+__device__ __forceinline__ void stage_tables(T* tab, const T* src, int len) {
+  const int4* s = reinterpret_cast<const int4*>(src);
+  int4* d = reinterpret_cast<int4*>(tab);
+  const int n = (int)((size_t)len * sizeof(T) / 16);
+#pragma unroll 4
+  for (int i = threadIdx.x; i < n; i += blockDim.x) d[i] = s[i];
+}
+// values of the tables that a constitutive kernel of variant NP keeps in shared memory
+template <typename T, int NP>
+__host__ __device__ inline int table_len(const MatDev<T>& M) {
+  return NP == 0 || NP == kLinearLaw ? 0 : (NP == kDirect ? M.rate_len : kRootTabs);
 }
 
 template <typename T>

@@ -51,7 +51,7 @@ cudaError_t launch_material_point_np(const MatDev<T>& M, long long nvox, const T
   if (nvox <= 0) return cudaSuccess;
   const int thr = 128;
   const long long grid = (nvox + thr - 1) / thr;
-  const size_t smem = (size_t)(kRootTabs) * sizeof(T);
+  const size_t smem = (size_t)table_len<T, NP>(M) * sizeof(T);
   cudaError_t e = set_smem<T>((const void*)k_material_point<T, NP>, smem);
   if (e != cudaSuccess) return e;
   k_material_point<T, NP><<<(unsigned)grid, thr, smem, s>>>(M, nvox, R, eps_n, eps, state, sigma, dt, nsub,
@@ -66,7 +66,7 @@ cudaError_t launch_material_point_vjp_np(const MatDev<T>& M, long long nvox, con
   if (nvox <= 0) return cudaSuccess;
   const int thr = 64;
   const long long grid = (nvox + thr - 1) / thr;
-  const size_t smem = (size_t)kRootTabs * sizeof(T);
+  const size_t smem = (size_t)table_len<T, NP>(M) * sizeof(T);
   cudaError_t e = set_smem<T>((const void*)k_material_point_vjp<T, NP>, smem);
   if (e != cudaSuccess) return e;
   k_material_point_vjp<T, NP><<<(unsigned)grid, thr, smem, s>>>(M, nvox, R, eps_n, eps, state, dt, nsub, sigma_b,
@@ -81,7 +81,7 @@ cudaError_t launch_adj_tangent_np(const MatDev<T>& M, long long nvox, const T* R
   if (nvox <= 0) return cudaSuccess;
   const int thr = 64;
   const long long grid = (nvox + thr - 1) / thr;
-  const size_t smem = (size_t)kRootTabs * sizeof(T);
+  const size_t smem = (size_t)table_len<T, NP>(M) * sizeof(T);
   cudaError_t e = set_smem<T>((const void*)k_adj_tangent<T, NP>, smem);
   if (e != cudaSuccess) return e;
   k_adj_tangent<T, NP><<<(unsigned)grid, thr, smem, s>>>(M, nvox, R, eps_n, eps, state, dt, nsub, (T)sd[0], (T)sd[1],
@@ -227,6 +227,15 @@ size_t line_group_smem(int n, int HC) {
 template <typename T>
 size_t zgreen_group_smem(int nz, int HC) {
   return line_group_smem<T>(nz, HC) + (size_t)HC * nz * sizeof(double);
+}
+
+template <typename T>
+cudaError_t launch_rate_table(T* out, bool two, const RateGrid& g0, const RateGrid& g1, double K0, double n0,
+                              double K1, double n1, double eta, cudaStream_t s) {
+  const int laws = two ? 2 : 1;
+  const int n = laws * RateFmt<T>::kSegs + (kExpTab<T> > 0 ? kExpTab<T> : laws);
+  k_rate_table<T><<<(n + 31) / 32, 32, 0, s>>>(out, two ? 1 : 0, g0, g1, K0, n0, K1, n1, eta);
+  return cudaGetLastError();
 }
 
 template <typename T>
@@ -494,6 +503,8 @@ cudaError_t launch_adj(int which, long long n, cudaStream_t s, const void* p0, c
 #define RVE_INSTANTIATE(T)                                                                                         \
   template cudaError_t launch_line<T>(const LineArgs<T>&, int, dim3, size_t, cudaStream_t);                       \
   template cudaError_t launch_zgreen<T>(const ZArgs<T>&, dim3, size_t, cudaStream_t);                             \
+  template cudaError_t launch_rate_table<T>(T*, bool, const RateGrid&, const RateGrid&, double, double, double,    \
+                                            double, double, cudaStream_t);                                         \
   template cudaError_t launch_shift<T>(C2<T>*, C2<T>*, long long, int, const double*, bool, cudaStream_t);        \
   template cudaError_t launch_xfft<T>(const XFftArgs<T>&, int, dim3, size_t, cudaStream_t);                       \
   template cudaError_t launch_to_double<T>(const T*, double*, long long, cudaStream_t, double);                   \

@@ -47,6 +47,16 @@ struct FftDim {
   int radix[12];
 };
 
+// Addressing of one law's direct rate table (rate_table.cuh): row (bits >> shift) - base with
+// the bits of a float argument or the high word of a double one, at most `last` - base; the
+// segment's midpoint has the bits (bits & mask) | half; lo is the float argument floor; off
+// the table's offset in the material's tables.
+template <typename T>
+struct RateLaw {
+  int shift, base, last, mask, half, off;
+  T lo;
+};
+
 // Material constants on the device (Sec. 3, Sec. 4), plus the reference medium.
 template <typename T>
 struct MatDev {
@@ -67,6 +77,11 @@ struct MatDev {
   // Hooke's law scaled by the slip systems' Schmid factor 1/sqrt6 (shear rows with their
   // factor 2): the stage's resolved stresses come from C_s : e directly
   T C11s, C12s, C13s, C33s, C44s2, C66s2;
+  // direct rate tables (variant kDirect): slip and twin laws, 1 / (nt - 1), and the values
+  // of all tables together
+  RateLaw<T> ls, lt;
+  T inv_ntm1;
+  int rate_len;
 };
 
 // Mixed-load controller data (always double).
@@ -114,6 +129,9 @@ constexpr double kRootSpan = 16.0;
 constexpr double kRootPerUnit = kRootIv / (2.0 * kRootSpan);
 constexpr int kRootTabLen = 2 * kRootIv;  // values per table
 constexpr int kRootTabs = 2 * kRootTabLen;  // slip systems' table, then the twin exponent's
+
+// Template value of the constitutive kernels' direct-table variant (rate_table.cuh).
+constexpr int kDirect = 3;
 
 // Template value of the x pass's linear-law mode (the adjoint solve): s = B eps - g per voxel.
 constexpr int kLinearLaw = 1;

@@ -132,7 +132,7 @@ __device__ __forceinline__ double mandel_w(int a) { return a < 3 ? 1.0 : 1.41421
 // load), so a grouped launch reads them at fixed parameter offsets.
 template <typename T>
 struct XCommon {
-  const T* root_tab;  // rate-root tables: kRootTabs values
+  const T* root_tab;  // rate tables: table_len values
   MatDev<T> M;
   LoadDev ld;
   T dt;
@@ -236,10 +236,10 @@ __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[32][kNumRed];
   __shared__ int s_last;
-  C2<T>* tw = reinterpret_cast<C2<T>*>(smem_raw);
+  T* tab = reinterpret_cast<T*>(smem_raw);  // rate tables (16-byte rows), then the FFT buffers
+  C2<T>* tw = reinterpret_cast<C2<T>*>(tab + table_len<T, NP>(k.M));
   C2<T>* b0 = tw + a.nx;
   C2<T>* b1 = b0 + 3 * a.L * a.xs;
-  T* tab = reinterpret_cast<T*>(b1 + 3 * a.L * a.xs);  // kRootTabs
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int nx = a.nx, H = a.H, half = nx / 2, xs = a.xs;
   const size_t NL = (size_t)a.ny * a.nz;
@@ -256,8 +256,7 @@ __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k
   }
 
   for (int i = tid; i < nx; i += nthr) tw[i] = a.tw[i];
-  if (NP != 0 && NP != kLinearLaw)
-    for (int i = tid; i < kRootTabs; i += nthr) tab[i] = k.root_tab[i];
+  stage_tables<T>(tab, k.root_tab, table_len<T, NP>(k.M));
   // pack component pairs (2p, 2p+1) of each line as one complex Hermitian-extended
   // sequence Z = A + iB, so one complex inverse FFT yields both real lines
   // (spectra are component-interleaved: entry (line, kx, c) at (line * H + kx) * 6 + c,
@@ -319,12 +318,7 @@ __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k
   #pragma unroll
       for (int c = 0; c < 6; ++c) epsn[c] = a.eps_n[c * nvox + vox];
       MPState<T> y;
-  #pragma unroll
-      for (int c = 0; c < 6; ++c) y.ep[c] = a.ep[c * nvox + vox];
-  #pragma unroll
-      for (int c = 0; c < 16; ++c) y.v[c] = a.v[c * nvox + vox];
-  #pragma unroll
-      for (int c = 0; c < 12; ++c) y.al[c] = a.al[c * nvox + vox];
+      load_voxel<T>(a.ep, a.v, a.al, nvox, vox, y);
       const uint32_t g = a.grain[vox];
   #pragma unroll
       for (int i = 0; i < 9; ++i) R[i] = a.Rg[(size_t)g * 9 + i];
@@ -335,7 +329,8 @@ __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k
       const size_t grp = ((size_t)line0 * nx + (size_t)(t - (tid & 31))) >> 5;
       const bool record = !COMMIT && a.flow != nullptr && it == 0;
       const bool check = COMMIT || a.flow == nullptr || it == 0 || a.flow[grp] == 0;
-      const bool flowed = mc_voxel<T, NP>(k.M, R, epsn, eps, y, k.dt, k.nsub, sig, tab, check);
+      const bool flowed =
+          mc_voxel_any<T, NP>(k.M, R, epsn, eps, y, k.dt, k.nsub, sig, tab, check, a.ep, a.v, a.al, nvox, vox);
       if (record) {
         const bool any = __any_sync(__activemask(), flowed);
         if ((tid & 31) == 0) a.flow[grp] = any ? 1 : 0;
@@ -449,7 +444,7 @@ __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k
 }
 
 template <typename T, bool COMMIT, int NP>
-__global__ void __launch_bounds__(kXThreads, XMinBlocks<T>::value) k_xpass(const XArgs<T> a) {
+__global__ void __launch_bounds__(kXThreads, XMinBlocks<T>::value) k_xpass(const __grid_constant__ XArgs<T> a) {
   xpass_cta<T, COMMIT, NP>(a, a.k, own_grid());
 }
 
@@ -1084,13 +1079,12 @@ __global__ void k_group_guard(const GuardGroup g, cudaGraphConditionalHandle con
 
 // ---------------------------------------------------------------- small kernels -----
 template <typename T, int NP>
-__global__ void k_material_point(const MatDev<T> M, long long nvox, const T* __restrict__ R,
+__global__ void k_material_point(const __grid_constant__ MatDev<T> M, long long nvox, const T* __restrict__ R,
                                  const T* __restrict__ eps_n, const T* __restrict__ eps, T* state,
                                  T* sigma, T dt, int nsub, const T* __restrict__ root_tab) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* tab = reinterpret_cast<T*>(smem_raw);  // kRootTabs
-  if (NP != 0)
-    for (int k = threadIdx.x; k < kRootTabs; k += blockDim.x) tab[k] = root_tab[k];
+  T* tab = reinterpret_cast<T*>(smem_raw);
+  stage_tables<T>(tab, root_tab, table_len<T, NP>(M));
   __syncthreads();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nvox) return;
@@ -1104,13 +1098,8 @@ __global__ void k_material_point(const MatDev<T> M, long long nvox, const T* __r
     e[c] = eps[c * n + i];
   }
   MPState<T> y;
-#pragma unroll
-  for (int c = 0; c < 6; ++c) y.ep[c] = state[c * n + i];
-#pragma unroll
-  for (int c = 0; c < 16; ++c) y.v[c] = state[(6 + c) * n + i];
-#pragma unroll
-  for (int c = 0; c < 12; ++c) y.al[c] = state[(22 + c) * n + i];
-  mc_voxel<T, NP>(M, r, en, e, y, dt, nsub, s, tab);
+  load_voxel<T>(state, state + 6 * n, state + 22 * n, n, (size_t)i, y);
+  mc_voxel_any<T, NP>(M, r, en, e, y, dt, nsub, s, tab, true, state, state + 6 * n, state + 22 * n, n, (size_t)i);
 #pragma unroll
   for (int c = 0; c < 6; ++c) state[c * n + i] = y.ep[c];
 #pragma unroll
