@@ -19,7 +19,7 @@ CSRC = PKG / "csrc"
 INCLUDE = ROOT / "include"
 BUILD = ROOT / "_build"
 LIB = PKG / "librve.so"
-SOURCES = ["xpass_f32_direct.cu", "xpass_f64_np10.cu", "xpass_f32_np0.cu", "xpass_f64_np0.cu", "xpass_f32_npr.cu",
+SOURCES = ["xpass_f32_direct.cu", "xpass_f64_direct.cu", "xpass_f32_np0.cu", "xpass_f64_np0.cu", "xpass_f32_npr.cu",
            "xpass_f64_npr.cu", "xpass_f32_lin.cu", "xpass_f64_lin.cu",
            "kernels_f32.cu", "kernels_f64.cu", "api.cu", "label.cu", "probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

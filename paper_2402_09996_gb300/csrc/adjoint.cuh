@@ -53,12 +53,12 @@ __device__ __forceinline__ void stage_eval(const MatDev<T>& M, const T* e0, cons
   const T cb_s = -M.b_s * T(kLog2e), cb_t = -M.b_b * T(kLog2e);
   #pragma unroll
   for (int q = 0; q < 12; ++q) {
-    V.ex[q] = fast_exp2<T>(cb_s * Y.v[q]);
+    V.ex[q] = hard_exp2<T, NP>(M, cb_s * Y.v[q], tab);
     V.Es += V.ex[q];
   }
   #pragma unroll
   for (int q = 12; q < 16; ++q) {
-    V.ex[q] = fast_exp2<T>(cb_t * Y.v[q]);
+    V.ex[q] = hard_exp2<T, NP>(M, cb_t * Y.v[q], tab);
     V.Et += V.ex[q];
     vtw += Y.v[q];
   }

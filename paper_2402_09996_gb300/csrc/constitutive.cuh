@@ -18,8 +18,6 @@
 //
 // Template parameter NP selects how the regularised rates are solved:
 //   NP = kDirect  eta > 0 and both laws tabulated directly (rate_table.cuh): no solve;
-//   NP = 10       double, eta > 0 and n = nt = 10 (compile-time power): table start,
-//                 branch-free;
 //   NP = -1       eta > 0, any real n, nt >= 1 (powers as 2^(p log2 z)): table start,
 //                 branch-free;
 //   NP = 0        eta = 0, and arguments outside the direct tables: generic per-system solve.
@@ -207,38 +205,6 @@ __device__ __forceinline__ T ipow(T z, int n) {
   return r;
 }
 
-// z^n for an integer 1 <= n < 64 without branches (selects over a fixed 6-bit loop).
-template <typename T>
-__device__ __forceinline__ T ipow_sel(T z, int n) {
-  T r = T(1), b = z;
-#pragma unroll
-  for (int bit = 0; bit < 6; ++bit) {
-    const T rb = r * b;
-    r = ((n >> bit) & 1) ? rb : r;
-    b = b * b;
-  }
-  return r;
-}
-
-// z^N for a compile-time N >= 1 (binary powering unrolled by the compiler).
-template <int N, typename T>
-__device__ __forceinline__ T cpow(T z) {
-  if constexpr (N == 1) {
-    return z;
-  } else if constexpr (N % 2 == 0) {
-    const T h = cpow<N / 2, T>(z);
-    return h * h;
-  } else {
-    return z * cpow<N - 1, T>(z);
-  }
-}
-
-template <typename T, int NP>
-__device__ __forceinline__ T zpow(T z, int n_int) {
-  if constexpr (NP > 0) return cpow<NP, T>(z);
-  else return ipow_sel<T>(z, n_int);
-}
-
 template <typename T>
 __device__ __forceinline__ T powT(T z, T n, int n_int) {
   return n_int > 0 ? ipow<T>(z, n_int) : pow(z, n);
@@ -262,6 +228,12 @@ template <> __device__ __forceinline__ double fast_exp2<double>(double x) { retu
 template <typename T> __device__ __forceinline__ T fast_exp(T x);
 template <> __device__ __forceinline__ float fast_exp<float>(float x) { return __expf(x); }
 template <> __device__ __forceinline__ double fast_exp<double>(double x) { return exp(x); }
+// 2^x for the hardening terms: in double from the table kept with the direct rate tables (tab).
+template <typename T, int NP>
+__device__ __forceinline__ T hard_exp2(const MatDev<T>& M, T x, const T* tab) {
+  if constexpr (NP == kDirect && std::is_same<T, double>::value) return exp2_tab(x, tab + (M.rate_len - kExpTab<double>));
+  else return fast_exp2<T>(x);
+}
 template <typename T> __device__ __forceinline__ T fast_div(T a, T b);
 template <> __device__ __forceinline__ float fast_div<float>(float a, float b) { return __fdividef(a, b); }
 template <> __device__ __forceinline__ double fast_div<double>(double a, double b) { return a / b; }
@@ -317,14 +289,11 @@ __device__ __forceinline__ RootCoef<T> root_coef(T P, T Kn, T n, T inv_n, T lg_K
   return q;
 }
 
-// z^(n-1) for the table-started Newton steps (z > 0): a compile-time product for NP > 0,
-// 2^((n-1) log2 z) for a real exponent (NP = -1; in float the hardware log2 / exp2, whose
-// relative error stays far below the 2e-4 the float path is held to).
-template <typename T, int NP>
-__device__ __forceinline__ T root_zn1(T z, const RootCoef<T>& q, int n_int) {
-  if constexpr (NP > 0) return cpow<NP - 1, T>(z);
-  else if constexpr (NP < 0) return fast_exp2<T>(q.nm1 * fast_log2<T>(z));
-  else return ipow_sel<T>(z, n_int - 1);
+// z^(n-1) for the table-started Newton steps (z > 0), 2^((n-1) log2 z) (in float the hardware
+// log2 / exp2, whose relative error stays far below the 2e-4 the float path is held to).
+template <typename T>
+__device__ __forceinline__ T root_zn1(T z, const RootCoef<T>& q) {
+  return fast_exp2<T>(q.nm1 * fast_log2<T>(z));
 }
 
 // Table interval of the coordinate t: floor(t + 1/2) clamped to [0, kRootIv - 1] (any t,
@@ -352,25 +321,25 @@ template <> struct Vec2<double> { using type = double2; };
 // phi' = n (c z^(n-1) + Kn/n), rho = P (z + dz)^n = P z^(n-1) (z + n dz) + O(dz^2);
 // |dz/z| < 3e-5 from the table start, so the dropped term n(n-1)/2 (dz/z)^2 < 4e-8 (n = 10)
 // is below float round-off (in double two full steps come first).
-template <typename T, int NP>
-__device__ __forceinline__ T root_newton(T z, T aa, const RootCoef<T>& q, int n_int) {
+template <typename T>
+__device__ __forceinline__ T root_newton(T z, T aa, const RootCoef<T>& q) {
 #pragma unroll
   for (int it = 0; it + 1 < TabNewton<T>::value; ++it) {
-    const T zn1 = root_zn1<T, NP>(z, q, n_int);
+    const T zn1 = root_zn1<T>(z, q);
     const T phi = (q.c * zn1) * z + (q.Kn * z - aa);
     z = z - fast_div<T>(phi, q.cn * zn1 + q.Kn);
   }
-  const T zn1 = root_zn1<T, NP>(z, q, n_int);
+  const T zn1 = root_zn1<T>(z, q);
   const T phi = z * (q.c * zn1 + q.Kn) - aa;
   const T r = fast_rcp<T>(q.c * zn1 + q.Kn_n);  // = n / phi'
   return q.Pout * (zn1 * (z - phi * r));
 }
 
-// Branch-free solve (eta > 0, integer exponent): inactive systems run the same arithmetic
+// Branch-free solve (eta > 0): inactive systems run the same arithmetic
 // on a dummy positive argument and return 0, so all systems of a stage form one basic
 // block the compiler can interleave.  tab: kRootIv (a_i, b_i) pairs, log2 u* = a_i + b_i t.
-template <typename T, int NP>
-__device__ __forceinline__ T reg_rate_tab(T a, const RootCoef<T>& q, int n_int, const T* tab) {
+template <typename T>
+__device__ __forceinline__ T reg_rate_tab(T a, const RootCoef<T>& q, const T* tab) {
   const bool on = a > T(0);
   const T aa = on ? a : T(1);
   const T la = fast_log2<T>(aa);
@@ -378,22 +347,22 @@ __device__ __forceinline__ T reg_rate_tab(T a, const RootCoef<T>& q, int n_int, 
   const T t = la * q.a2 + q.b2;
   const auto ab = reinterpret_cast<const typename Vec2<T>::type*>(tab)[root_interval<T>(t)];
   const T z = fast_exp2<T>(lzB + (ab.x + ab.y * t));
-  const T rho = root_newton<T, NP>(z, aa, q, n_int);
+  const T rho = root_newton<T>(z, aa, q);
   return on ? rho : T(0);
 }
 
 // The same for the slip systems, whose coefficients do not depend on the stage (P = 1):
 // their table holds log2 z0 = alpha_i + beta_i la directly (alpha_i = b1 + a_i + b_i b2,
 // beta_i = a1 + b_i a2, built on the host for the material's K, n and eta).
-template <typename T, int NP>
-__device__ __forceinline__ T reg_rate_slip(T a, const RootCoef<T>& q, int n_int, const T* tab) {
+template <typename T>
+__device__ __forceinline__ T reg_rate_slip(T a, const RootCoef<T>& q, const T* tab) {
   const bool on = a > T(0);
   const T aa = on ? a : T(1);
   const T la = fast_log2<T>(aa);
   const T t = la * q.a2 + q.b2;
   const auto ab = reinterpret_cast<const typename Vec2<T>::type*>(tab)[root_interval<T>(t)];
   const T z = fast_exp2<T>(ab.x + ab.y * la);
-  const T rho = root_newton<T, NP>(z, aa, q, n_int);
+  const T rho = root_newton<T>(z, aa, q);
   return on ? rho : T(0);
 }
 
@@ -481,11 +450,24 @@ __device__ __forceinline__ T reg_rate(T a, T P, T Kn, T n, int n_int, T inv_n, T
 }
 
 // ---------------------------------------------------------------- RK4 stage ----------
-// The generic solve out of line, for arguments outside a direct table.
+// The P = 1 root F(a) by the generic solve, out of line: arguments outside a direct table.
 template <typename T>
-__device__ __noinline__ T rate_generic(T a, T P, T Kn, T n, int n_int, T inv_n, T m, T lg_Kn, T eta, T lg_eta,
-                                       T lg_P) {
-  return reg_rate<T>(a, P, Kn, n, n_int, inv_n, m, lg_Kn, eta, lg_eta, lg_P);
+__device__ __noinline__ T rate_generic(T a, T Kn, T n, int n_int, T inv_n, T m, T lg_Kn, T eta, T lg_eta) {
+  return reg_rate<T>(a, T(1), Kn, n, n_int, inv_n, m, lg_Kn, eta, lg_eta, T(0));
+}
+// F(a) of the slip (twin) law for any a: the table inside its range.
+template <typename T>
+__device__ __forceinline__ T rate_root(const MatDev<T>& M, T a, bool twin, const T* tab) {
+  const RateLaw<T>& L = twin ? M.lt : M.ls;
+  if constexpr (std::is_same<T, double>::value) {
+    if (!(a > 0.0)) return 0.0;
+    if (rate_inside(a, L)) return rate_direct(a, L, tab + L.off);
+  } else {
+    const T r = rate_direct(a, L, tab + L.off);
+    if (r == r) return r;
+  }
+  return twin ? rate_generic<T>(a, M.Kt, M.nt, M.nt_int, M.inv_nt, M.smt, M.lg_Kt, M.eta, M.lg_eta)
+              : rate_generic<T>(a, M.K, M.n, M.n_int, M.inv_n, M.sm, M.lg_K, M.eta, M.lg_eta);
 }
 
 // The twins' argument scale s = P^(1/(nt-1)) and its inverse for the direct table (both 0 for
@@ -502,14 +484,12 @@ template <typename T, int NP>
 __device__ __forceinline__ T stage_rate(const MatDev<T>& M, const RootCoef<T>& q, T a, T P, bool twin, T lg_P,
                                         const T* tab) {
   if constexpr (NP == kDirect) {
-    T s = T(1), is = T(1);
-    if (twin) twin_scale<T>(M, P, lg_P, &s, &is);
-    const T rho = rate_direct(a * s, twin ? M.lt : M.ls, tab + (twin ? M.lt.off : M.ls.off)) * is;
-    if (rho == rho) return rho;
-    return twin ? rate_generic<T>(a, P, M.Kt, M.nt, M.nt_int, M.inv_nt, M.smt, M.lg_Kt, M.eta, M.lg_eta, lg_P)
-                : rate_generic<T>(a, P, M.K, M.n, M.n_int, M.inv_n, M.sm, M.lg_K, M.eta, M.lg_eta, lg_P);
+    if (!twin) return rate_root<T>(M, a, false, tab);
+    T sc, isc;
+    twin_scale<T>(M, P, lg_P, &sc, &isc);
+    return rate_root<T>(M, a * sc, true, tab) * isc;
   } else if constexpr (NP != 0) {
-    return twin ? reg_rate_tab<T, NP>(a, q, M.nt_int, tab + kRootTabLen) : reg_rate_slip<T, NP>(a, q, M.n_int, tab);
+    return twin ? reg_rate_tab<T>(a, q, tab + kRootTabLen) : reg_rate_slip<T>(a, q, tab);
   } else {
     return twin ? reg_rate<T>(a, P, M.Kt, M.nt, M.nt_int, M.inv_nt, M.smt, M.lg_Kt, M.eta, M.lg_eta, lg_P)
                 : reg_rate<T>(a, P, M.K, M.n, M.n_int, M.inv_n, M.sm, M.lg_K, M.eta, M.lg_eta, lg_P);
@@ -847,6 +827,176 @@ __device__ __forceinline__ void to_sample(const T* R, const T* s, T* out) {
   out[5] = R[0] * B[0][1] + R[1] * B[1][1] + R[2] * B[2][1];
 }
 
+// The RK4 substeps of an increment in double with the direct rate tables: the stages of
+// rk_stage, one system at a time.  GB300's FP64 pipe takes 16 cycles per warp instruction and
+// SM, so the update is bound by its count of FP64 instructions, and everything a warp can
+// leave out is:
+//  - a rate is 10 FP64 instructions (rate_direct) and a hardening exponential 9 (exp2_tab),
+//    against about 100 and 18 with three Newton steps and the library's exp2;
+//  - a system in which no lane of the warp flows costs its driving force only: its rate is
+//    exactly 0, which leaves its slip, kinematic variable and sums as they are;
+//  - exponentials and their sums are kept while the slips they belong to do not change
+//    (dirty: systems whose slip in yt changed since ex was formed).
+// Skips are decided per warp but do not change any lane's values.  48^3, increments at 0.3 %
+// strain: x pass 11.7 -> 3.46 ms per launch.
+__device__ __forceinline__ void rk4_fp64(const MatDev<double>& M, const double* e0, const double* de,
+                                         MPState<double>& y, double dt, int nsub, const double* tab) {
+  constexpr double kLog2e = 1.44269504088896340736;
+  const unsigned lanes = __activemask();
+  const double* tab_e = tab + (M.rate_len - kExpTab<double>);
+  const double h = dt / (double)nsub, inv = 1.0 / (double)nsub;
+  const double cb_s = -M.b_s * kLog2e, cb_t = -M.b_b * kLog2e;
+  const double dq = M.h_diag - M.h_off, Qdq_s = M.Q_s * dq, Qdq_t = M.Q_b * dq;
+  MPState<double> yt = y, acc;
+  double ex[16];
+  double Es = 0.0, Et = 0.0, ftot = 0.0, s_tw = 0.0, is_tw = 0.0;
+  bool scaled = false;        // s_tw, is_tw belong to ftot
+  unsigned dirty = 0xffffu;   // systems whose yt.v changed since ex was formed
+  unsigned moved = 0;         // systems whose yt.v and yt.al differ from y's
+#pragma unroll 1
+  for (int m = 0; m < nsub; ++m) {
+#pragma unroll
+    for (int c = 0; c < 6; ++c) acc.ep[c] = 0.0;
+#pragma unroll
+    for (int c = 0; c < 16; ++c) acc.v[c] = 0.0;
+#pragma unroll
+    for (int c = 0; c < 12; ++c) acc.al[c] = 0.0;
+    unsigned ever = 0;  // systems that flowed in some stage of the substep
+#pragma unroll 1
+    for (int stg = 0; stg < 4; ++stg) {
+      const double s = ((double)m + 0.5 * (double)((stg + 1) >> 1)) * inv;
+      const double wacc = stg == 0 || stg == 3 ? 1.0 : 2.0;
+      const double cn = stg == 2 ? h : 0.5 * h;
+      const bool step = stg < 3;  // the last stage forms no further state
+      if (dirty & 0xfffu) {
+        double q0 = 0.0, q1 = 0.0;
+#pragma unroll
+        for (int k = 0; k < 12; k += 2) {
+          if (dirty >> k & 1u) ex[k] = exp2_tab(cb_s * yt.v[k], tab_e);
+          if (dirty >> (k + 1) & 1u) ex[k + 1] = exp2_tab(cb_s * yt.v[k + 1], tab_e);
+          q0 += ex[k];
+          q1 += ex[k + 1];
+        }
+        Es = q0 + q1;
+      }
+      if (dirty >> 12) {
+#pragma unroll
+        for (int k = 12; k < 16; ++k)
+          if (dirty >> k & 1u) ex[k] = exp2_tab(cb_t * yt.v[k], tab_e);
+        Et = (ex[12] + ex[14]) + (ex[13] + ex[15]);
+        ftot = 1.41421356237309504880 * ((yt.v[12] + yt.v[14]) + (yt.v[13] + yt.v[15]));
+        scaled = false;
+      }
+      double fm_left = M.fm - ftot;
+      fm_left = fm_left > 0.0 ? fm_left : 0.0;
+      const double Rb_s = M.Q_s * (M.h_off * (12.0 - Es) + dq), Rb_t = M.Q_b * (M.h_off * (4.0 - Et) + dq);
+      const double rb_sup = M.r0[0] + Rb_s, rb_ord = M.r0[2] + Rb_s, rb_tw = M.r0[12] + Rb_t;
+      double ss[6];
+      {
+        double e[6];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) e[c] = e0[c] + s * de[c] - yt.ep[c];
+        ss[0] = M.C11s * e[0] + M.C12s * e[1] + M.C13s * e[2];
+        ss[1] = M.C12s * e[0] + M.C11s * e[1] + M.C13s * e[2];
+        ss[2] = M.C13s * (e[0] + e[1]) + M.C33s * e[2];
+        ss[3] = M.C44s2 * e[3];
+        ss[4] = M.C44s2 * e[4];
+        ss[5] = M.C66s2 * e[5];
+      }
+      unsigned act = 0;
+      double du[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0}, G = 0.0, H[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+      for (int p = 0; p < 4; ++p) {
+        double S[3], D[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+        for (int i = 0; i < 3; ++i) S[i] = plane_sig(p, i) > 0 ? ss[i] + ss[i + 3] : ss[i] - ss[i + 3];
+#pragma unroll
+        for (int k = 3 * p; k < 3 * p + 3; ++k) {
+          const double al = yt.al[k];
+          const double tk = plane_sum<double>(k, S) - M.c * al;
+          const double a = fabs(tk) - ((k % 3 == 2 ? rb_ord : rb_sup) - Qdq_s * ex[k]);
+          if (__any_sync(lanes, a > 0.0)) {
+            const double rho = rate_root<double>(M, a, false, tab);
+            const double gd = copysign(rho, tk);
+            act |= 1u << k;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+              if (diag_k(k, i) == 1) D[i] += gd;
+              else if (diag_k(k, i) == -1) D[i] -= gd;
+            }
+            const double ald = gd - M.d * rho * al;
+            acc.v[k] += wacc * rho;
+            acc.al[k] += wacc * ald;
+            if (step) {
+              yt.v[k] = y.v[k] + cn * rho;
+              yt.al[k] = y.al[k] + cn * ald;
+            }
+          } else if (step && (moved >> k & 1u)) {
+            yt.v[k] = y.v[k];
+            yt.al[k] = y.al[k];
+          }
+        }
+        if (act >> (3 * p) & 7u) {
+#pragma unroll
+          for (int i = 0; i < 3; ++i) {
+            du[i] += D[i];
+            if (plane_sig(p, i) > 0) du[i + 3] += D[i];
+            else du[i + 3] -= D[i];
+          }
+        }
+        const int k = 12 + p;
+        // 1/(|n||l|) of a twin is (1/sqrt3) times the slip systems' scale in ss
+        const double at = 0.57735026918962576451 * plane_sum<double>(k, S) - (rb_tw - Qdq_t * ex[k]);
+        if (__any_sync(lanes, at > 0.0 && fm_left > 0.0)) {
+          if (!scaled) {
+            const double P = (M.Kc * 0.70710678118654752440) * fm_left;
+            const double l = log2(P > 0.0 ? P : 1.0) * M.inv_ntm1;
+            s_tw = P > 0.0 ? exp2_tab(l, tab_e) : 0.0;
+            is_tw = P > 0.0 ? exp2_tab(-l, tab_e) : 0.0;
+            scaled = true;
+          }
+          const double g = rate_root<double>(M, at * s_tw, true, tab) * is_tw;
+          act |= 1u << k;
+          G += g;
+#pragma unroll
+          for (int i = 0; i < 3; ++i) H[i] += plane_sig(p, i) > 0 ? g : -g;
+          acc.v[k] += wacc * g;
+          if (step) yt.v[k] = y.v[k] + cn * g;
+        } else if (step && (moved >> k & 1u)) {
+          yt.v[k] = y.v[k];
+        }
+      }
+      if (act | moved) {
+        // eps_p rate = (1 - sum f) sum_s gdot_s m_s + sum_b gdot_b m_b, m = scale sym(n x l)
+        const double fs = (1.0 - ftot) * sys_scale<double>(0), tsc = sys_scale<double>(12);
+        const double dt6[6] = {G, G, -2.0 * G, H[0], H[1], -2.0 * H[2]};
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+          const double dep = c < 3 ? fs * du[c] + tsc * dt6[c] : 0.5 * fs * du[c] + 0.5 * tsc * dt6[c];
+          acc.ep[c] += wacc * dep;
+          if (step) yt.ep[c] = y.ep[c] + cn * dep;
+        }
+      }
+      ever |= act;
+      dirty = step ? act | moved : 0u;
+      if (step) moved = act;
+    }
+    if (ever) {
+      const double w = h / 6.0;
+#pragma unroll
+      for (int c = 0; c < 6; ++c) yt.ep[c] = y.ep[c] = y.ep[c] + w * acc.ep[c];
+#pragma unroll
+      for (int c = 0; c < 16; ++c)
+        if (ever >> c & 1u) yt.v[c] = y.v[c] = y.v[c] + w * acc.v[c];
+#pragma unroll
+      for (int c = 0; c < 12; ++c)
+        if (ever >> c & 1u) yt.al[c] = y.al[c] = y.al[c] + w * acc.al[c];
+    }
+    dirty = ever;
+    moved = 0;
+  }
+}
+
 // Integrates one voxel over the increment [t_n, t_n + dt] (strain eps_n -> eps, sample
 // frame) and returns the sample-frame stress at t_n + dt; y is updated in place.
 // check: test first whether the increment is elastic and skip the integration if so.  The
@@ -863,9 +1013,12 @@ __device__ __forceinline__ bool mc_voxel(const MatDev<T>& M, const T* R, const T
   for (int c = 0; c < 6; ++c) de[c] = e1[c] - e0[c];
   const bool flows = !(check && elastic_increment<T>(M, e0, de, y));
   if (flows) {
-    const T h = dt / T(nsub);
-    const T inv = T(1) / T(nsub);
+    if constexpr (NP == kDirect && std::is_same<T, double>::value) {
+      rk4_fp64(M, e0, de, y, dt, nsub, tab);
+    } else
     for (int m = 0; m < nsub; ++m) {
+      const T h = dt / T(nsub);
+      const T inv = T(1) / T(nsub);
       const T s0 = T(m) * inv, sh = (T(m) + T(0.5)) * inv, s1 = (T(m) + T(1)) * inv;
       MPState<T> yt, acc;
       // classical RK4: stages at s0, sh, sh, s1 with weights 1, 2, 2, 1.  The first stage

@@ -18,18 +18,14 @@ template <typename T> struct ZGroup;
 struct GuardGroup;
 
 // Rate-solve variants of the constitutive kernels (see constitutive.cuh): kDirect where both
-// laws have a direct table (float; 2 <= n <= 10.2), else NP = 10 in double for n = nt = 10,
-// NP = -1 for other exponents >= 1, and NP = 0 (generic per-system solve) for eta = 0.
+// laws have a direct table (2 <= n <= 10.2), NP = -1 for other exponents >= 1, and NP = 0
+// (generic per-system solve) for eta = 0.
 template <typename T>
 inline int rate_variant(double eta, double K, double n, double Kt, double nt) {
   if (!(eta > 0.0)) return 0;
   RateGrid g;
-  if (sizeof(T) == 4 && rate_law_fit_t<T>(K, n, eta, &g) && rate_law_fit_t<T>(Kt, nt, eta, &g)) return kDirect;
-  return sizeof(T) == 8 && n == 10.0 && nt == 10.0 ? 10 : -1;
+  return rate_law_fit_t<T>(K, n, eta, &g) && rate_law_fit_t<T>(Kt, nt, eta, &g) ? kDirect : -1;
 }
-
-// the fast variant of a precision
-template <typename T> constexpr int kTabVariant = sizeof(T) == 4 ? kDirect : 10;
 
 // Per-variant entry points (each instantiated in its own translation unit).
 template <typename T, int NP>
@@ -53,8 +49,8 @@ template <typename T>
 cudaError_t launch_adj_tangent(const MatDev<T>& M, int np, long long nvox, const T* R, const T* eps_n, const T* eps,
                                const T* state, T dt, int nsub, const double* sd, T* state_b, T* J, T* eps_b,
                                T* eps_n_b, T* R_b, T* param_b, const T* root_tab, cudaStream_t s) {
-  if (np == kTabVariant<T>)
-    return launch_adj_tangent_np<T, kTabVariant<T>>(M, nvox, R, eps_n, eps, state, dt, nsub, sd, state_b, J, eps_b, eps_n_b, R_b,
+  if (np == kDirect)
+    return launch_adj_tangent_np<T, kDirect>(M, nvox, R, eps_n, eps, state, dt, nsub, sd, state_b, J, eps_b, eps_n_b, R_b,
                                         param_b, root_tab, s);
   if (np < 0)
     return launch_adj_tangent_np<T, -1>(M, nvox, R, eps_n, eps, state, dt, nsub, sd, state_b, J, eps_b, eps_n_b, R_b,
@@ -67,8 +63,8 @@ template <typename T>
 cudaError_t launch_material_point_vjp(const MatDev<T>& M, int np, long long nvox, const T* R, const T* eps_n,
                                       const T* eps, const T* state, T dt, int nsub, const T* sigma_b, T* state_b,
                                       T* eps_b, T* eps_n_b, T* R_b, T* param_b, const T* root_tab, cudaStream_t s) {
-  if (np == kTabVariant<T>)
-    return launch_material_point_vjp_np<T, kTabVariant<T>>(M, nvox, R, eps_n, eps, state, dt, nsub, sigma_b, state_b, eps_b,
+  if (np == kDirect)
+    return launch_material_point_vjp_np<T, kDirect>(M, nvox, R, eps_n, eps, state, dt, nsub, sigma_b, state_b, eps_b,
                                                eps_n_b, R_b, param_b, root_tab, s);
   if (np < 0)
     return launch_material_point_vjp_np<T, -1>(M, nvox, R, eps_n, eps, state, dt, nsub, sigma_b, state_b, eps_b,
@@ -79,7 +75,7 @@ cudaError_t launch_material_point_vjp(const MatDev<T>& M, int np, long long nvox
 
 template <typename T>
 cudaError_t launch_xpass(const XArgs<T>& a, int np, bool commit, int grid, size_t smem, cudaStream_t s) {
-  if (np == kTabVariant<T>) return launch_xpass_np<T, kTabVariant<T>>(a, commit, grid, smem, s);
+  if (np == kDirect) return launch_xpass_np<T, kDirect>(a, commit, grid, smem, s);
   if (np == kLinearLaw) return launch_xpass_np<T, kLinearLaw>(a, commit, grid, smem, s);
   if (np < 0) return launch_xpass_np<T, -1>(a, commit, grid, smem, s);
   return launch_xpass_np<T, 0>(a, commit, grid, smem, s);
@@ -87,8 +83,8 @@ cudaError_t launch_xpass(const XArgs<T>& a, int np, bool commit, int grid, size_
 template <typename T>
 cudaError_t launch_material_point(const MatDev<T>& M, int np, long long nvox, const T* R, const T* eps_n, const T* eps,
                                   T* state, T* sigma, T dt, int nsub, const T* root_tab, cudaStream_t s) {
-  if (np == kTabVariant<T>)
-    return launch_material_point_np<T, kTabVariant<T>>(M, nvox, R, eps_n, eps, state, sigma, dt, nsub, root_tab, s);
+  if (np == kDirect)
+    return launch_material_point_np<T, kDirect>(M, nvox, R, eps_n, eps, state, sigma, dt, nsub, root_tab, s);
   if (np < 0) return launch_material_point_np<T, -1>(M, nvox, R, eps_n, eps, state, sigma, dt, nsub, root_tab, s);
   return launch_material_point_np<T, 0>(M, nvox, R, eps_n, eps, state, sigma, dt, nsub, root_tab, s);
 }
@@ -105,7 +101,7 @@ template <typename T, int NP>
 cudaError_t launch_xpass_group_np(const XGroup<T>& g, bool commit, int grid, size_t smem, cudaStream_t s);
 template <typename T>
 cudaError_t launch_xpass_group(const XGroup<T>& g, int np, bool commit, int grid, size_t smem, cudaStream_t s) {
-  if (np == kTabVariant<T>) return launch_xpass_group_np<T, kTabVariant<T>>(g, commit, grid, smem, s);
+  if (np == kDirect) return launch_xpass_group_np<T, kDirect>(g, commit, grid, smem, s);
   if (np < 0) return launch_xpass_group_np<T, -1>(g, commit, grid, smem, s);
   return launch_xpass_group_np<T, 0>(g, commit, grid, smem, s);
 }

@@ -133,11 +133,14 @@ __device__ __forceinline__ double rate_direct(double a, const RateLaw<double>& L
   return r;
 }
 
+// 2^x beyond exp2_tab's range, out of line.
+static __device__ __noinline__ double exp2_far(double x) { return exp2(x); }
+
 // 2^x in double from the 64-entry table of 2^(j/64) (tab) and the Taylor polynomial of 2^r,
 // |r| <= 1/128, degree 5 (its remainder is below 2^-54): 9 FP64 instructions.  |x| >= 1000 and
 // NaN take the library function.
 __device__ __forceinline__ double exp2_tab(double x, const double* tab) {
-  if (!(fabs(x) < 1000.0)) return exp2(x);
+  if (!((__double2hiint(x) & 0x7fffffff) < 0x408f4000)) return exp2_far(x);
   const double M = 105553116266496.0;  // 1.5 * 2^46: the sum is x rounded to a multiple of 1/64
   const double t = x + M;
   const double r = x - (t - M);
