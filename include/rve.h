@@ -355,7 +355,7 @@ rve_status rve_label_voronoi(int nx, int ny, int nz, int n_parent, const double*
  * trigger the implicit device-wide synchronisation of those calls (latency-critical
  * loops, other work in flight on the device), and library code embedded where
  * allocation is forbidden.  This variant keeps its scratch (seeds, normals, centroid sums
- * of up to RVE_NOALLOC_MAX_PARENTS parents, about 470 KB) in one static device array that
+ * of up to RVE_NOALLOC_MAX_PARENTS parents, about 550 KB) in one static device array that
  * every GPU loading this library holds until the process exits.
  *   Inputs and output as rve_label_voronoi, except that grain_id_out must be a device
  *   pointer (nx*ny*nz labels).  n_parent > RVE_NOALLOC_MAX_PARENTS -> RVE_ERR_INVALID_ARG.
