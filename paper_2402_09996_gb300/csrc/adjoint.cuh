@@ -553,6 +553,7 @@ __global__ void k_material_point_vjp(const MatDev<T> M, long long nvox, const T*
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* tab = reinterpret_cast<T*>(smem_raw);
   stage_tables<T>(tab, root_tab, table_len<T, NP>(M));
+  stage_wait();
   __syncthreads();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nvox) return;
@@ -597,6 +598,7 @@ __global__ void k_adj_tangent(const MatDev<T> M, long long nvox, const T* __rest
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* tab = reinterpret_cast<T*>(smem_raw);
   stage_tables<T>(tab, root_tab, table_len<T, NP>(M));
+  stage_wait();
   __syncthreads();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nvox) return;

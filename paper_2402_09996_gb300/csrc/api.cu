@@ -324,8 +324,16 @@ rve_status dalloc(rve_s* h, void** p, size_t bytes) {
   *p = nullptr;
   if (bytes == 0) bytes = 16;
   if (h->opt.alloc) {
-    *p = h->opt.alloc(bytes, h->opt.alloc_ctx);
-    if (!*p) return fail(h, RVE_ERR_OOM, "allocator callback returned NULL");
+    void* q = h->opt.alloc(bytes, h->opt.alloc_ctx);
+    if (q && (uintptr_t)q % 16 != 0) {
+      // the kernels use 16-byte accesses and asynchronous copies: ask for room to align
+      h->opt.free(q, h->opt.alloc_ctx);
+      q = h->opt.alloc(bytes + 16, h->opt.alloc_ctx);
+    }
+    if (!q) return fail(h, RVE_ERR_OOM, "allocator callback returned NULL");
+    *p = (void*)(((uintptr_t)q + 15) / 16 * 16);
+    h->owned.push_back(q);
+    return RVE_OK;
   } else {
     cudaError_t e = cudaMalloc(p, bytes);
     if (e != cudaSuccess) {
@@ -335,6 +343,13 @@ rve_status dalloc(rve_s* h, void** p, size_t bytes) {
   }
   h->owned.push_back(*p);
   return RVE_OK;
+}
+
+// Gives the most recent allocation back.
+void drop_last(rve_s* h) {
+  if (h->opt.free) h->opt.free(h->owned.back(), h->opt.alloc_ctx);
+  else cudaFree(h->owned.back());
+  h->owned.pop_back();
 }
 
 // Per-launch event timing (opt.timing): a launch records into an event slot; after the
@@ -555,6 +570,31 @@ size_t z_smem(const rve_s* h, int hc) {
   return (size_t)(h->nz + 12 * hc * (h->nz + 1)) * 2 * sizeof(T) + (size_t)hc * h->nz * sizeof(double);
 }
 
+// x lines per CTA of the x pass (128 threads; a CTA's L nx voxels take r = ceil(L nx / 128)
+// rounds).  The pass is bound by the constitutive update, so the busiest SM's rounds,
+// ceil(CTAs / 152) r, set its time; among equals, the fewest rounds in sequence, counting half
+// a round per CTA for its transforms and table copy (`resident` CTAs share an SM), then the
+// larger L.  At most 5 rounds, which keeps 3 float CTAs per SM in shared memory.  Measured x
+// passes: 48^3 FP64 L = 8 2.06 ms (7: 2.78, 5: 2.53, 16: 2.50), 32^3 FP64 L = 4 0.72 (8: 0.86),
+// 20^3 FP64 L = 6 0.41 (7: 0.70), 64^3 FP32 L = 4 141 us (8: 156, 2: 150), 96^3 L = 4 383
+// (5: 401), 128^3 L = 4 804 (3: 824, 5: 815, 2: 863), 160^3 L = 4 1536 (3: 1598, 5: 1596).
+int x_lines_per_cta(int nx, long long NL, int resident) {
+  const long long sms = 152, thr = x_threads();
+  int best = 1;
+  long long cost = -1, seq = -1;
+  for (int L = 1; L <= NL; ++L) {
+    const long long r = ((long long)L * nx + thr - 1) / thr, n = (NL + L - 1) / L;
+    if (r > 5 && L > 1) break;
+    const long long c = (n + sms - 1) / sms * r, q = (2 * r + 1) * ((n + sms * resident - 1) / (sms * resident));
+    if (cost < 0 || c < cost || (c == cost && q <= seq)) {
+      best = L;
+      cost = c;
+      seq = q;
+    }
+  }
+  return best;
+}
+
 template <typename T>
 rve_status alloc_fields(rve_s* h) {
   const size_t spec = (size_t)6 * h->NL * h->H * 2 * sizeof(T);
@@ -580,15 +620,7 @@ rve_status alloc_fields(rve_s* h) {
     RVE_CUDA(h, cudaMemsetAsync(h->flow, 0, nflow, h->stream));
   }
   // launch geometry
-  // x lines per CTA: enough to give every thread a voxel, up to 4 voxels per thread (a
-  // thread then integrates voxels of several lines, which evens out the elastic/plastic
-  // work between the CTA's warps) while keeping at least 2 CTAs per SM
-  {
-    const long long fill = (x_threads() + h->nx - 1) / h->nx;
-    const long long most = std::max<long long>(1, 4LL * x_threads() / h->nx);
-    const long long keep = std::max<long long>(1, h->NL / (2 * 152));
-    h->L = (int)std::max(fill, std::min(most, keep));
-  }
+  h->L = x_lines_per_cta(h->nx, h->NL, h->opt.precision == RVE_FP64 ? 2 : 3);
   h->xgrid = (int)((h->NL + h->L - 1) / h->L);
   // x sequences in shared memory: odd stride nx + 1 for the register transforms of the
   // lengths with a two-step split (conflict-free steps), nx for the Stockham passes
@@ -1790,9 +1822,7 @@ rve_status get_field_t(rve_s* h, int which, int dtype, void* dst, size_t bytes, 
   if (dtype == RVE_DTYPE_F32 && !on_dev) {
     rve_status s = dalloc(h, &tmp32, n * sizeof(float));
     if (s) {
-      h->owned.pop_back();
-      if (h->opt.free) h->opt.free(tmp, h->opt.alloc_ctx);
-      else cudaFree(tmp);
+      drop_last(h);
       return s;
     }
   }
@@ -1807,10 +1837,7 @@ rve_status get_field_t(rve_s* h, int which, int dtype, void* dst, size_t bytes, 
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   for (void* t : {tmp32, tmp}) {  // the last allocations first, as dalloc recorded them
-    if (!t) continue;
-    h->owned.pop_back();
-    if (h->opt.free) h->opt.free(t, h->opt.alloc_ctx);
-    else cudaFree(t);
+    if (t) drop_last(h);
   }
   if (e != cudaSuccess) return cuda_fail(h, e, "get_fields");
   return RVE_OK;

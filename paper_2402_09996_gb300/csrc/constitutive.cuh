@@ -1096,15 +1096,19 @@ __device__ __forceinline__ bool mc_voxel_any(const MatDev<T>& M, const T* R, con
   return flows;
 }
 
-// Copies the rate tables (a multiple of 16 bytes) to shared memory; no barrier.
+// Starts the copy of the rate tables (16-byte aligned, a multiple of 16 bytes) to shared memory;
+// stage_wait and a barrier complete it.
 template <typename T>
 __device__ __forceinline__ void stage_tables(T* tab, const T* src, int len) {
-  const int4* s = reinterpret_cast<const int4*>(src);
-  int4* d = reinterpret_cast<int4*>(tab);
+  const unsigned d = (unsigned)__cvta_generic_to_shared(tab);
   const int n = (int)((size_t)len * sizeof(T) / 16);
 #pragma unroll 4
-  for (int i = threadIdx.x; i < n; i += blockDim.x) d[i] = s[i];
+  for (int i = threadIdx.x; i < n; i += blockDim.x)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + 16u * i),
+                 "l"(reinterpret_cast<const char*>(src) + 16 * (size_t)i)
+                 : "memory");
 }
+__device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 // values of the tables that a constitutive kernel of variant NP keeps in shared memory
 template <typename T, int NP>
 __host__ __device__ inline int table_len(const MatDev<T>& M) {

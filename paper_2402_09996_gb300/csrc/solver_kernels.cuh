@@ -229,8 +229,49 @@ constexpr int kXThreads = 128;
 template <typename T> struct XMinBlocks { static constexpr int value = 1; };
 template <> struct XMinBlocks<float> { static constexpr int value = 3; };
 
+// Two adjacent complex values (a component pair of a spectral point) with 16-byte accesses.
+template <typename T> struct SpecPair { C2<T> a, b; };
+template <typename T>
+__device__ __forceinline__ SpecPair<T> load_pair(const C2<T>* p) {
+  SpecPair<T> r;
+  if constexpr (sizeof(T) == 4) {
+    const float4 f = *reinterpret_cast<const float4*>(p);
+    r.a = mk<T>(f.x, f.y);
+    r.b = mk<T>(f.z, f.w);
+  } else {
+    r.a = p[0];
+    r.b = p[1];
+  }
+  return r;
+}
+template <typename T>
+__device__ __forceinline__ void store_pair(C2<T>* p, C2<T> a, C2<T> b) {
+  if constexpr (sizeof(T) == 4) {
+    *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
+  } else {
+    p[0] = a;
+    p[1] = b;
+  }
+}
+
+// Fetches into L2 the rows base[c nvox + vox0 ..] (count values each, c < comps) that the CTA
+// reads later.
+template <typename T>
+__device__ __forceinline__ void prefetch_rows(const T* base, int comps, size_t nvox, size_t vox0, int count, int tid,
+                                              int nthr) {
+  constexpr int kPer = 128 / (int)sizeof(T);
+  const unsigned lines = (unsigned)((count + kPer - 1) / kPer), m = recip_small(lines);
+  for (unsigned i = tid; i < comps * lines; i += nthr) {
+    const unsigned c = div_small(i, lines, m);
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(base + c * nvox + vox0 + (i - c * lines) * kPer));
+  }
+}
+
 // One CTA of the x pass (see the file header) at grid place `cta`; k holds a.k or the
-// group's common arguments.
+// group's common arguments.  Before the constitutive update a CTA would wait in turn for its
+// spectrum, its tables and its state; the tables' copy to shared memory and the prefetch of
+// the state's rows are issued first, and a thread's loads of the spectrum (up to kPack
+// component pairs) are all in flight at once.  128^3 FP32 x pass: 817 -> 788 us, with n_sub = 1 396 -> 374 us.
 template <typename T, bool COMMIT, int NP>
 __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k, const Cta& cta) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -255,28 +296,56 @@ __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k
     spec_in = k == 0 ? a.cand[0] : ((k & 1) ? a.cand[1] : a.cand[2]);
   }
 
-  for (int i = tid; i < nx; i += nthr) tw[i] = a.tw[i];
   stage_tables<T>(tab, k.root_tab, table_len<T, NP>(k.M));
+  for (int i = tid; i < nx; i += nthr) tw[i] = a.tw[i];
   // pack component pairs (2p, 2p+1) of each line as one complex Hermitian-extended
   // sequence Z = A + iB, so one complex inverse FFT yields both real lines
   // (spectra are component-interleaved: entry (line, kx, c) at (line * H + kx) * 6 + c,
   // so consecutive threads read consecutive component pairs of the CTA's lines)
-  for (int w = tid; w < 3 * nl * H; w += nthr) {
-    const int p = w % 3;
-    const int r = w / 3;
-    const int xi = r % H, l = r / H;
-    const int q = p * nl + l;
-    const size_t e0 = (((size_t)line0 + l) * H + xi) * 6 + 2 * p;
-    C2<T> A = spec_in[e0];
-    C2<T> B = spec_in[e0 + 1];
-    if (xi == 0 || xi == half) {
-      A.y = T(0);
-      B.y = T(0);
+  const unsigned m3 = recip_small(3u), mH = recip_small((unsigned)H), mnx = recip_small((unsigned)nx);
+  const int npair = 3 * nl * H;
+  {
+    constexpr int kPack = sizeof(T) == 4 ? 8 : 4;
+    const C2<T>* src = spec_in + (size_t)line0 * H * 6;
+    bool fetched = false;
+    for (int w0 = tid; w0 < npair; w0 += kPack * nthr) {
+      SpecPair<T> v[kPack];
+#pragma unroll
+      for (int j = 0; j < kPack; ++j)
+        if (w0 + j * nthr < npair) v[j] = load_pair<T>(src + 2 * (size_t)(w0 + j * nthr));
+      if (!fetched) {
+        fetched = true;
+        const size_t vox0 = (size_t)line0 * nx;
+        if constexpr (NP == kLinearLaw) {
+          prefetch_rows<T>(a.lin_B, 36, nvox, vox0, nl * nx, tid, nthr);
+          prefetch_rows<T>(a.lin_g, 6, nvox, vox0, nl * nx, tid, nthr);
+        } else {
+          prefetch_rows<T>(a.eps_n, 6, nvox, vox0, nl * nx, tid, nthr);
+          prefetch_rows<T>(a.ep, 6, nvox, vox0, nl * nx, tid, nthr);
+          prefetch_rows<T>(a.v, 16, nvox, vox0, nl * nx, tid, nthr);
+          prefetch_rows<T>(a.al, 12, nvox, vox0, nl * nx, tid, nthr);
+          prefetch_rows<uint32_t>(a.grain, 1, nvox, vox0, nl * nx, tid, nthr);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < kPack; ++j) {
+        const int w = w0 + j * nthr;
+        if (w < npair) {
+          const int r = (int)div_small((unsigned)w, 3u, m3), p = w - 3 * r;
+          const int l = (int)div_small((unsigned)r, (unsigned)H, mH), xi = r - l * H;
+          C2<T> A = v[j].a, B = v[j].b;
+          if (xi == 0 || xi == half) {
+            A.y = T(0);
+            B.y = T(0);
+          }
+          C2<T>* seq = b0 + (size_t)(p * nl + l) * xs;
+          seq[xi] = mk<T>(A.x - B.y, A.y + B.x);
+          if (xi > 0 && xi < half) seq[nx - xi] = mk<T>(A.x + B.y, B.x - A.y);
+        }
+      }
     }
-    C2<T>* seq = b0 + (size_t)q * xs;
-    seq[xi] = mk<T>(A.x - B.y, A.y + B.x);
-    if (xi > 0 && xi < half) seq[nx - xi] = mk<T>(A.x + B.y, B.x - A.y);
   }
+  stage_wait();
   __syncthreads();
   C2<T>* res = xlines_fft<T, +1>(b0, b1, a.dx, 3 * nl, xs, tw, tid, nthr);
   C2<T>* oth = (res == b0) ? b1 : b0;
@@ -288,7 +357,7 @@ __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k
   // most in float) and added to the FP64 block sum once
   T sacc[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
   for (int t = tid; t < nl * nx; t += nthr) {
-    const int l = t / nx, x = t - l * nx;
+    const int l = (int)div_small((unsigned)t, (unsigned)nx, mnx), x = t - l * nx;
     const size_t vox = ((size_t)line0 + l) * nx + x;
     T eps[6], epsn[6], sig[6], R[9];
 #pragma unroll
@@ -376,18 +445,16 @@ __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k
     __syncthreads();
     C2<T>* out = xlines_fft<T, -1>(res, oth, a.dx, 3 * nl, xs, tw, tid, nthr);
     // unpack: A = (Z_k + conj Z_{n-k}) / 2, B = (Z_k - conj Z_{n-k}) / (2i)
-    for (int w = tid; w < 3 * nl * H; w += nthr) {
-      const int p = w % 3;
-      const int r = w / 3;
-      const int xi = r % H, l = r / H;
+    C2<T>* dst = a.spec_out + (size_t)line0 * H * 6;
+    for (int w = tid; w < npair; w += nthr) {
+      const int r = (int)div_small((unsigned)w, 3u, m3), p = w - 3 * r;
+      const int l = (int)div_small((unsigned)r, (unsigned)H, mH), xi = r - l * H;
       const int q = p * nl + l;
       const C2<T> Z = out[(size_t)q * xs + xi];
       const C2<T> Zm = out[(size_t)q * xs + (xi == 0 ? 0 : nx - xi)];
       const C2<T> A = mk<T>(T(0.5) * (Z.x + Zm.x), T(0.5) * (Z.y - Zm.y));
       const C2<T> B = mk<T>(T(0.5) * (Z.y + Zm.y), T(-0.5) * (Z.x - Zm.x));
-      const size_t e0 = (((size_t)line0 + l) * H + xi) * 6 + 2 * p;
-      a.spec_out[e0] = A;
-      a.spec_out[e0 + 1] = B;
+      store_pair<T>(dst + 2 * (size_t)w, A, B);
     }
   }
   // trial iterations sum the 6 stress components (in-warp in the field precision); the
@@ -1085,6 +1152,7 @@ __global__ void k_material_point(const __grid_constant__ MatDev<T> M, long long 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* tab = reinterpret_cast<T*>(smem_raw);
   stage_tables<T>(tab, root_tab, table_len<T, NP>(M));
+  stage_wait();
   __syncthreads();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nvox) return;
