@@ -288,8 +288,7 @@ struct rve_s {
   double lin_sref = 0.0;  // source scale of the adjoint fixed point (floor of the error norms)
   // FFT tile autotuner (opt.autotune): runs once, before the first increment
   bool tuned = false;
-  IterStatus* st_tune = nullptr;  // scratch status and history for timing the z pass
-  double* hist_tune = nullptr;
+  IterStatus* st_tune = nullptr;  // scratch status for timing the z pass
 };
 
 namespace {
@@ -563,7 +562,7 @@ rve_status upload_tables(rve_s* h) {
 // the z pass (the same + HC*nz residual terms).
 template <typename T>
 size_t y_smem(const rve_s* h, int hc) {
-  return (size_t)(h->ny + 12 * hc * (h->ny + 1)) * 2 * sizeof(T);
+  return std::max((size_t)(h->ny + 12 * hc * (h->ny + 1)) * 2 * sizeof(T), (size_t)kSideSmem);
 }
 template <typename T>
 size_t z_smem(const rve_s* h, int hc) {
@@ -652,7 +651,6 @@ rve_status alloc_fields(rve_s* h) {
   if ((s = dalloc(h, (void**)&h->dhist, (size_t)2 * max_iter * sizeof(double)))) return s;
   if ((s = dalloc(h, (void**)&h->st_tune, sizeof(IterStatus)))) return s;
   RVE_CUDA(h, cudaMemsetAsync(h->st_tune, 0, sizeof(IterStatus), h->stream));
-  if ((s = dalloc(h, (void**)&h->hist_tune, 2 * sizeof(double)))) return s;
   return RVE_OK;
 }
 
@@ -747,10 +745,23 @@ XArgs<T> x_args(rve_s* h, const void* in, void* out, int it) {
     a.lin_g = (const T*)h->lin_g;
     if (!out) a.eps_n = (T*)h->lin_mu;  // the linear-law commit writes the solution field here
   }
-  // mixed load
+  a.k.dt = (T)h->dt;
+  a.k.nsub = h->opt.n_sub > 0 ? h->opt.n_sub : default_nsub(h->dt);
+  a.partial = h->partial;
+  a.counter = h->counter;
+  a.st = h->st;
+  a.it = it;
+  a.done = out ? &h->st->done : nullptr;  // the commit (no output spectrum) always runs
+  return a;
+}
+
+int max_iter_of(const rve_s* h) { return h->opt.max_iter > 0 ? h->opt.max_iter : 1000; }
+
+// Mixed-load data of the device's macroscopic update (mean_update).
+LoadDev load_dev(const rve_s* h) {
   double M0[36];
   c0_mandel(h->lam0, h->mu0, M0);
-  LoadDev& ld = a.k.ld;
+  LoadDev ld;
   std::memset(&ld, 0, sizeof(ld));
   int fi[6], nf = 0;
   for (int c = 0; c < 6; ++c) {
@@ -768,13 +779,23 @@ XArgs<T> x_args(rve_s* h, const void* in, void* out, int it) {
     for (int i = 0; i < nf; ++i)
       for (int j = 0; j < nf; ++j) ld.Minv[fi[i] * 6 + fi[j]] = Mff[i * nf + j];
   }
-  a.k.dt = (T)h->dt;
-  a.k.nsub = h->opt.n_sub > 0 ? h->opt.n_sub : default_nsub(h->dt);
+  return ld;
+}
+
+// The small reduction that a y pass does beside its transforms.
+SideArgs side_args(rve_s* h, int kind, int it) {
+  SideArgs a{};
+  a.kind = kind;
   a.partial = h->partial;
-  a.counter = h->counter;
+  a.count = kind == kSideMean ? (size_t)h->xgrid : (size_t)h->ny * h->H;
   a.st = h->st;
+  a.inv_nvox = 1.0 / (double)h->nvox;
   a.it = it;
-  a.done = out ? &h->st->done : nullptr;  // the commit (no output spectrum) always runs
+  if (kind == kSideMean) a.ld = load_dev(h);
+  a.conv.tol = h->opt.tol;
+  a.conv.fixed_iters = h->opt.fixed_iters;
+  a.conv.max_iter = max_iter_of(h);
+  a.conv.hist = h->dhist;
   return a;
 }
 
@@ -814,14 +835,8 @@ ZArgs<T> z_args(rve_s* h, void* spec, const void* Pp, void* Po, int it) {
   a.lam0 = (T)h->lam0;
   a.mu0 = (T)h->mu0;
   a.invN = (T)(1.0 / (double)h->nvox);
-  a.conv.tol = h->opt.tol;
-  a.conv.fixed_iters = h->opt.fixed_iters;
-  a.conv.max_iter = h->opt.max_iter > 0 ? h->opt.max_iter : 1000;
-  a.conv.hist = h->dhist;
-  a.conv.s_ref = h->lin_mode ? h->lin_sref : 0.0;
   a.done = &h->st->done;
   a.partial = h->partial;
-  a.counter = h->counter;
   a.st = h->st;
   a.it = it;
   return a;
@@ -877,8 +892,6 @@ struct Rotation {
   int p_in(int it) const { return it == 0 ? p0 : p_out(it - 1); }
 };
 
-int max_iter_of(const rve_s* h) { return h->opt.max_iter > 0 ? h->opt.max_iter : 1000; }
-
 int np_of(const rve_s* h) {
   const rve_material& m = h->mat;
   if (h->lin_mode) return kLinearLaw;
@@ -887,7 +900,7 @@ int np_of(const rve_s* h) {
 
 // One fixed-point iteration (x pass, forward y, z + Green, inverse y) on stream s:
 // strain spectrum si -> so, tau_hat spectra pi -> po.  it < 0: the kernels take the
-// iteration index from the device (graph mode) and the residual kernel clears `cond`
+// iteration index from the device (graph mode) and the residual's CTA clears `cond`
 // once it decides.  `slot` >= 0 brackets the launches with timing events.
 template <typename T>
 rve_status enqueue_one(rve_s* h, cudaStream_t s, int it, int si, int so, int pi, int po,
@@ -901,19 +914,21 @@ rve_status enqueue_one(rve_s* h, cudaStream_t s, int it, int si, int so, int pi,
   RVE_CUDA(h, launch_xpass<T>(xa, np, false, h->xgrid, xsmem_total(h), s));
   if (timed) tstop(h, 4 * slot + 0);
   LineArgs<T> ya = y_args<T>(h, h->spec[so]);
+  ya.side = side_args(h, kSideMean, it);
   if (timed) tstart(h, 4 * slot + 1, RVE_K_YFWD);
-  RVE_CUDA(h, launch_line<T>(ya, -1, dim3(ygrid_x, h->nz), h->ysmem, s));
+  RVE_CUDA(h, launch_line<T>(ya, -1, dim3(ygrid_x, h->nz + 1), h->ysmem, s));
   if (timed) tstop(h, 4 * slot + 1);
   ZArgs<T> za = z_args<T>(h, h->spec[so], h->P[pi], h->P[po], it);
-  if (cond) {
-    za.has_cond = 1;
-    za.cond = *cond;
-  }
   if (timed) tstart(h, 4 * slot + 2, RVE_K_ZGREEN);
   RVE_CUDA(h, launch_zgreen<T>(za, dim3(zgrid_x, h->ny), h->zsmem, s));
   if (timed) tstop(h, 4 * slot + 2);
+  ya.side = side_args(h, kSideResid, it);
+  if (cond) {
+    ya.side.has_cond = 1;
+    ya.side.cond = *cond;
+  }
   if (timed) tstart(h, 4 * slot + 3, RVE_K_YINV);
-  RVE_CUDA(h, launch_line<T>(ya, +1, dim3(ygrid_x, h->nz), h->ysmem, s));
+  RVE_CUDA(h, launch_line<T>(ya, +1, dim3(ygrid_x, h->nz + 1), h->ysmem, s));
   if (timed) tstop(h, 4 * slot + 3);
   return RVE_OK;
 }
@@ -1090,10 +1105,6 @@ rve_status tune_tiles(rve_s* h) {
       za.HC = hc;
       za.st = h->st_tune;
       za.done = &h->st_tune->done;
-      za.conv.hist = h->hist_tune;
-      za.conv.fixed_iters = 1 << 30;  // never decides
-      za.conv.max_iter = 1 << 30;
-      za.has_cond = 0;
       const dim3 grid((h->H + hc - 1) / hc, h->ny);
       float ms = 0.f;
       e = timed([&] { return launch_zgreen<T>(za, grid, sm, s); }, &ms);
@@ -1338,7 +1349,7 @@ bool groupable(rve_s* const* hs, int n) {
 template <typename T>
 struct GroupIter {
   XGroup<T> x;
-  LineGroup<T> y;
+  LineGroup<T> y, yi;  // forward and inverse y pass
   ZGroup<T> z;
   int xgrid = 0, ygrid = 0, zgrid = 0;
   size_t xsmem = 0, ysmem = 0, zsmem = 0;
@@ -1361,14 +1372,15 @@ void group_iter_args(const std::vector<rve_s*>& hs, int which, GroupIter<T>& g) 
     g.xgrid += h->xgrid;
     g.xsmem = std::max(g.xsmem, xsmem_total(h));
     g.y.m[m] = y_args<T>(h, h->spec[so]);
+    g.y.m[m].side = side_args(h, kSideMean, -1);
+    g.yi.m[m] = g.y.m[m];
+    g.yi.m[m].side = side_args(h, kSideResid, -1);  // the group guard ends the loop
     const int ygx = (h->H + h->yHC - 1) / h->yHC;
-    g.y.start[m] = g.ygrid;
-    g.y.gx[m] = ygx;
-    g.ygrid += ygx * h->nz;
+    g.y.start[m] = g.yi.start[m] = g.ygrid;
+    g.y.gx[m] = g.yi.gx[m] = ygx;
+    g.ygrid += ygx * (h->nz + 1);
     g.ysmem = std::max(g.ysmem, line_group_smem<T>(h->ny, h->yHC));
-    ZArgs<T> za = z_args<T>(h, h->spec[so], h->P[pi], h->P[po], -1);
-    za.has_cond = 0;  // the group guard ends the loop
-    g.z.m[m] = za;
+    g.z.m[m] = z_args<T>(h, h->spec[so], h->P[pi], h->P[po], -1);
     const int zgx = (h->H + h->zHC - 1) / h->zHC;
     g.z.start[m] = g.zgrid;
     g.z.gx[m] = zgx;
@@ -1376,9 +1388,9 @@ void group_iter_args(const std::vector<rve_s*>& hs, int which, GroupIter<T>& g) 
     g.zsmem = std::max(g.zsmem, zgreen_group_smem<T>(h->nz, h->zHC));
   }
   g.x.k = g.x.m[0].k;
-  g.x.n = g.y.n = g.z.n = n;
+  g.x.n = g.y.n = g.yi.n = g.z.n = n;
   g.x.start[n] = g.xgrid;
-  g.y.start[n] = g.ygrid;
+  g.y.start[n] = g.yi.start[n] = g.ygrid;
   g.z.start[n] = g.zgrid;
 }
 
@@ -1387,7 +1399,7 @@ cudaError_t group_iteration(const GroupIter<T>& g, int np, cudaStream_t s) {
   cudaError_t e = launch_xpass_group<T>(g.x, np, false, g.xgrid, g.xsmem, s);
   if (e == cudaSuccess) e = launch_line_group<T>(g.y, -1, g.ygrid, g.ysmem, s);
   if (e == cudaSuccess) e = launch_zgreen_group<T>(g.z, g.zgrid, g.zsmem, s);
-  if (e == cudaSuccess) e = launch_line_group<T>(g.y, +1, g.ygrid, g.ysmem, s);
+  if (e == cudaSuccess) e = launch_line_group<T>(g.yi, +1, g.ygrid, g.ysmem, s);
   return e;
 }
 

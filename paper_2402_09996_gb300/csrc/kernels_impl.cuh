@@ -3,6 +3,8 @@
 // constitutive kernels, one rate-solve variant per translation unit).
 #pragma once
 
+#include <algorithm>
+
 #include "adjoint.cuh"
 #include "launch.h"
 #include "solver_kernels.cuh"
@@ -222,7 +224,7 @@ template <typename T>
 size_t line_group_smem(int n, int HC) {
   const size_t pencil = ((size_t)n + (size_t)6 * HC * (n + 1)) * sizeof(C2<T>);
   const size_t stock = ((size_t)n + (size_t)2 * 6 * HC * (n + 1)) * sizeof(C2<T>);
-  return HC <= pencil_max_hc(n) ? pencil : stock;
+  return std::max(HC <= pencil_max_hc(n) ? pencil : stock, (size_t)kSideSmem);
 }
 template <typename T>
 size_t zgreen_group_smem(int nz, int HC) {

@@ -98,6 +98,7 @@ struct IterStatus {
   double E[2][6];       // E^(i) in slot i%2 (tensor components)
   double sig_mean[6];   // <sigma>^(i)
   double cF;            // stress-constraint error
+  double inv_norm;      // 1 / (nvox max(|<sigma>|, s_ref)), 0 when that norm is 0
   double res_sum;       // sum_xi w |kappa . sigma_hat|^2
   double e_eq;          // equilibrium error
   double eff[4];        // commit: <sigma_eq>, <f_beta>, <v^s>, unused
@@ -115,7 +116,6 @@ struct ConvDev {
   int fixed_iters;  // > 0: stop after exactly this many iterations
   int max_iter;
   double* hist;     // 2 * max_iter: (e_eq, c_F) of every iteration of the increment
-  double s_ref;     // floor of the mean-stress norm in the relative errors (0: none)
 };
 
 constexpr int kNumRed = 9;  // reduction slots per CTA

@@ -6,13 +6,14 @@
 // Between iterations S holds the strain with x still in Fourier space and y, z in
 // real space ("x-spectral" form).  One iteration:
 //   k_xpass   inverse x-FFT -> eps(x) -> per-voxel MC update -> sigma, tau = sigma - C0:eps
-//             -> forward x-FFT (out of place); sums of sigma (per thread and in-warp in
-//             the field precision, across warps and CTAs in FP64); the last CTA forms
-//             <sigma>, the stress-constraint error and the mixed-load update.
-//   k_line_pencil / k_line   forward y-FFT (in place)
+//             -> forward x-FFT (out of place); sums of sigma per CTA (per thread and
+//             in-warp in the field precision, across warps in FP64).
+//   k_line_pencil / k_line   forward y-FFT (in place); beside it one CTA adds the sums (FP64)
+//             and forms <sigma>, the stress-constraint error and the mixed-load update.
 //   k_zgreen  forward z-FFT -> eps_hat = -Gamma0(kappa):tau_hat / N, eps_hat(0) = E,
-//             equilibrium residual (FP64 sums) -> inverse z-FFT (in place)
-//   k_line_pencil / k_line   inverse y-FFT (in place)
+//             equilibrium residual per (ky, kx) column -> inverse z-FFT (in place)
+//   k_line_pencil / k_line   inverse y-FFT (in place); beside it one CTA adds the residual
+//             (FP64) and decides convergence.
 #pragma once
 
 #include "constitutive.cuh"
@@ -59,7 +60,8 @@ __device__ __forceinline__ Cta own_grid() {
   return Cta{blockIdx.x, blockIdx.y, blockIdx.x + gridDim.x * blockIdx.y, gridDim.x * gridDim.y};
 }
 
-// Stores this CTA's sums and returns true (in all threads) in the CTA that finished last.
+// Stores this CTA's sums and returns true (in all threads) in the CTA that finished last (the
+// commit, which no pass follows).
 template <int NV>
 __device__ __forceinline__ bool publish_partial(double* v, double* partial, unsigned int* counter,
                                                 double (*red)[kNumRed], int* s_last, const Cta& cta) {
@@ -75,14 +77,13 @@ __device__ __forceinline__ bool publish_partial(double* v, double* partial, unsi
   return *s_last != 0;
 }
 
-// publish_partial for NV sums held in the field precision T: the in-warp shuffle tree runs
-// in T (in float, the adds of GB300's slow FP64 pipe are kept out of every thread), the
-// warp sums are converted and added across warps in FP64.  For T = double this is
-// publish_partial's arithmetic.
+// Stores NV sums of the CTA (nw <= 4 warps), held per thread in T, at partial[i * stride]: the
+// in-warp shuffle tree runs in T (in float, the adds of GB300's slow FP64 pipe are kept out of
+// every thread), the warp sums are converted and added across warps in FP64.
 template <typename T, int NV>
-__device__ __forceinline__ bool publish_partial_t(const T* s, double* partial, unsigned int* counter,
-                                                  double (*red)[kNumRed], int* s_last, const Cta& cta) {
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+__device__ __forceinline__ void store_partial(const T* s, double* partial, size_t stride, double (*red)[kNumRed],
+                                              int nw) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   T v[NV];
 #pragma unroll
   for (int i = 0; i < NV; ++i) v[i] = s[i];
@@ -94,21 +95,40 @@ __device__ __forceinline__ bool publish_partial_t(const T* s, double* partial, u
 #pragma unroll
     for (int i = 0; i < NV; ++i) red[wid][i] = (double)v[i];
   __syncthreads();
-  if (wid == 0) {
-    double w[NV];
-#pragma unroll
-    for (int i = 0; i < NV; ++i) w[i] = lane < nw ? red[lane][i] : 0.0;
-    warp_sum<NV>(w);
-    if (lane == 0) {
-#pragma unroll
-      for (int i = 0; i < NV; ++i) partial[(size_t)cta.lin * kNumRed + i] = w[i];
-      __threadfence();
-      const unsigned int prev = atomicAdd(counter, 1u);
-      *s_last = (prev == cta.count - 1) ? 1 : 0;
+  if (threadIdx.x < NV) {
+    const int i = threadIdx.x;
+    const double r1 = nw > 1 ? red[1][i] : 0.0, r2 = nw > 2 ? red[2][i] : 0.0, r3 = nw > 3 ? red[3][i] : 0.0;
+    partial[i * stride] = (red[0][i] + r2) + (r1 + r3);
+  }
+}
+
+// Sums of NV rows of n values (row i at p + i n) in an order that does not depend on the block
+// size (a multiple of 32): row i is cut into kSplit contiguous parts, one per virtual warp,
+// whose lane l takes the part's values l, l + 32, ... with four accumulators; a shuffle tree
+// adds the lanes.  A warp instruction of the FP64 pipe takes 64 cycles on its scheduler, so
+// the rows go to different warps and a tree adds one value.  The NV * kSplit sums are left in
+// red (row i's parts at red[i kSplit ..]); contains a barrier at its end.
+template <int NV, int kSplit>
+__device__ __forceinline__ void rows_total(const double* p, size_t n, double* red) {
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int w = threadIdx.x >> 5; w < NV * kSplit; w += nw) {
+    const size_t part = (n + kSplit - 1) / kSplit, b0 = (w % kSplit) * part;
+    const double* r = p + (size_t)(w / kSplit) * n;
+    const size_t end = b0 + part < n ? b0 + part : n;
+    double q0 = 0.0, q1 = 0.0, q2 = 0.0, q3 = 0.0;
+    size_t b = b0 + lane;
+    for (; b + 96 < end; b += 128) {
+      q0 += r[b];
+      q1 += r[b + 32];
+      q2 += r[b + 64];
+      q3 += r[b + 96];
     }
+    for (; b < end; b += 32) q0 += r[b];
+    double v = (q0 + q1) + (q2 + q3);
+    warp_sum<1>(&v);
+    if (lane == 0) red[w] = v;
   }
   __syncthreads();
-  return *s_last != 0;
 }
 
 // Deterministic grand total of all CTAs' partials (fixed assignment and tree order).
@@ -127,14 +147,13 @@ __device__ __forceinline__ void total_partials(const double* partial, double* v,
 __device__ __forceinline__ double mandel_w(int a) { return a < 3 ? 1.0 : 1.41421356237309504880; }
 
 // ---------------------------------------------------------------- x pass -----------
-// The x pass's arguments that do not depend on the grid: material, load, increment and
-// the rate-root tables.  RVEs stepped as one group share them (identical material and
+// The x pass's arguments that do not depend on the grid: material, increment and the rate
+// tables.  RVEs stepped as one group share them (identical material and
 // load), so a grouped launch reads them at fixed parameter offsets.
 template <typename T>
 struct XCommon {
   const T* root_tab;  // rate tables: table_len values
   MatDev<T> M;
-  LoadDev ld;
   T dt;
   int nsub;
 };
@@ -275,7 +294,7 @@ __device__ __forceinline__ void prefetch_rows(const T* base, int comps, size_t n
 template <typename T, bool COMMIT, int NP>
 __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k, const Cta& cta) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double red[32][kNumRed];
+  __shared__ double red[kXThreads / 32][kNumRed];
   __shared__ int s_last;
   T* tab = reinterpret_cast<T*>(smem_raw);  // rate tables (16-byte rows), then the FFT buffers
   C2<T>* tw = reinterpret_cast<C2<T>*>(tab + table_len<T, NP>(k.M));
@@ -457,54 +476,30 @@ __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k
       store_pair<T>(dst + 2 * (size_t)w, A, B);
     }
   }
-  // trial iterations sum the 6 stress components (in-warp in the field precision); the
-  // commit and the linear-law mode all slots in FP64
-  constexpr bool kSix = !COMMIT && NP != kLinearLaw;
-  bool last;
-  if constexpr (kSix) last = publish_partial_t<T, 6>(sacc, a.partial, a.counter, red, &s_last, cta);
-  else last = publish_partial<kNumRed>(acc, a.partial, a.counter, red, &s_last, cta);
-  if (last) {
-    if constexpr (kSix) total_partials<6>(a.partial, acc, red, cta.count);
-    else total_partials<kNumRed>(a.partial, acc, red, cta.count);
+  // Trial iterations leave the CTA's 6 stress sums (in-warp in the field precision; the
+  // linear law's in FP64) to the forward y pass, which forms the mean and the mixed-load
+  // update (mean_update) beside its transforms: a CTA that waited for its stores and a ticket
+  // held its SM for 6500 cycles, and the last one added all sums alone (36 us at 128^3).
+  if constexpr (!COMMIT) {
+    double* out = a.partial + cta.lin;
+    if constexpr (NP == kLinearLaw) store_partial<double, 6>(acc, out, cta.count, red, nthr >> 5);
+    else store_partial<T, 6>(sacc, out, cta.count, red, nthr >> 5);
+  } else if (publish_partial<kNumRed>(acc, a.partial, a.counter, red, &s_last, cta)) {
+    total_partials<kNumRed>(a.partial, acc, red, cta.count);
     if (tid == 0) {
       IterStatus* st = a.st;
       const double inv = 1.0 / (double)a.nvox;
-      double S[6];
       int bad = 0;
       for (int c = 0; c < 6; ++c) {
-        S[c] = acc[c] * inv;
-        st->sig_mean[c] = S[c];
-        bad |= !isfinite(S[c]);
+        const double S = acc[c] * inv;
+        st->sig_mean[c] = S;
+        bad |= !isfinite(S);
       }
-      if (COMMIT) {
-        st->eff[0] = acc[6] * inv;
-        st->eff[1] = acc[7] * inv * 0.25;
-        st->eff[2] = acc[8] * inv / 12.0;
-        bad |= !isfinite(acc[6]) | !isfinite(acc[7]) | !isfinite(acc[8]);
-      } else {
-        // mixed-load update of the free components (Mandel form)
-        const LoadDev& ld = k.ld;
-        double miss[6], nm = 0.0, ns = 0.0;
-        for (int c = 0; c < 6; ++c) {
-          const double sm = S[c] * mandel_w(c);
-          miss[c] = ld.free_mask[c] ? sm - ld.Sigma_m[c] : 0.0;
-          nm += miss[c] * miss[c];
-          ns += sm * sm;
-        }
-        st->cF = ld.any_free ? sqrt(nm) / fmax(sqrt(ns), ld.s_ref) : 0.0;
-        const double* Ec = st->E[it & 1];
-        double* En = st->E[(it + 1) & 1];
-        for (int c = 0; c < 6; ++c) {
-          double em = Ec[c] * mandel_w(c);
-          if (ld.free_mask[c]) {
-            double corr = 0.0;
-            for (int b = 0; b < 6; ++b) corr += ld.Minv[c * 6 + b] * miss[b];
-            em -= corr;
-          }
-          En[c] = em / mandel_w(c);
-        }
-      }
-      st->nan_flag |= bad ? (COMMIT ? 4 : 1) : 0;
+      st->eff[0] = acc[6] * inv;
+      st->eff[1] = acc[7] * inv * 0.25;
+      st->eff[2] = acc[8] * inv / 12.0;
+      bad |= !isfinite(acc[6]) | !isfinite(acc[7]) | !isfinite(acc[8]);
+      st->nan_flag |= bad ? 4 : 0;
       *a.counter = 0u;
     }
   }
@@ -523,6 +518,103 @@ __global__ void __launch_bounds__(kXThreads, XMinBlocks<T>::value) k_xpass(const
 // h0 = bx * HC.  The solver's spectra are component-interleaved (NC = 6,
 // hstride = 6: each (j, kx chunk) row is HC * 6 contiguous values); the stand-alone FFT
 // entry points use component-major spectra (NC = 1, hstride = 1).
+//
+// The solver's passes carry the iteration's small reductions in one CTA of an extra first row
+// of their grid (side != kSideNone; the transform of row o = by - 1): the forward y pass the
+// x pass's stress sums (mean_update), the inverse y pass the z pass's residual sums and the
+// convergence decision (resid_update), so that they run beside the transforms.
+enum { kSideNone = 0, kSideMean = 1, kSideResid = 2 };
+constexpr int kSideSmem = 12 * sizeof(double);  // dynamic shared memory the side work needs
+
+struct SideArgs {
+  int kind;
+  const double* partial;
+  size_t count;  // x-pass CTAs (6 rows of them) or (ky, kx) columns
+  IterStatus* st;
+  double inv_nvox;
+  int it;  // iteration index; < 0: st->it_dev, advanced by resid_update (graph mode)
+  LoadDev ld;
+  ConvDev conv;
+  int has_cond;  // graph mode: clear the loop condition once the increment is decided
+  cudaGraphConditionalHandle cond;
+};
+
+// Mean stress, stress-constraint error and mixed-load update of the free components (Mandel
+// form) from the x pass's per-CTA sums; lane c of warp 0 holds component c.
+static __device__ __noinline__ void mean_update(const SideArgs& a, double* red) {
+  rows_total<6, 2>(a.partial, a.count, red);
+  if (threadIdx.x >= 32) return;
+  const int lane = threadIdx.x, c = lane < 6 ? lane : 0;
+  IterStatus* st = a.st;
+  const LoadDev& ld = a.ld;
+  const int it = a.it >= 0 ? a.it : st->it_dev;
+  const double S = (red[2 * c] + red[2 * c + 1]) * a.inv_nvox;
+  const double w = mandel_w(c), sm = S * w;
+  const double miss = lane < 6 && ld.free_mask[c] ? sm - ld.Sigma_m[c] : 0.0;
+  double n2[2] = {miss * miss, lane < 6 ? sm * sm : 0.0};
+#pragma unroll
+  for (int off = 4; off > 0; off >>= 1)
+#pragma unroll
+    for (int i = 0; i < 2; ++i) n2[i] += __shfl_xor_sync(0xffffffffu, n2[i], off);
+  double corr = 0.0;
+#pragma unroll
+  for (int b = 0; b < 6; ++b) corr += ld.Minv[c * 6 + b] * __shfl_sync(0xffffffffu, miss, b);
+  const unsigned bad = __ballot_sync(0xffffffffu, lane < 6 && !isfinite(S));
+  if (lane < 6) {
+    st->sig_mean[c] = S;
+    double em = st->E[it & 1][c] * w;
+    if (ld.free_mask[c]) em -= corr;
+    st->E[(it + 1) & 1][c] = c < 3 ? em : em * 0.70710678118654752440;
+  }
+  // norms of the misfit (lane 0) and of the mean stress, floored (lane 1)
+  double nr = sqrt(lane == 0 ? n2[0] : n2[1]);
+  if (lane != 0) nr = fmax(nr, ld.s_ref);
+  const double nm = __shfl_sync(0xffffffffu, nr, 1);
+  if (lane == 0) {
+    st->cF = ld.any_free ? nr / nm : 0.0;
+    if (bad) st->nan_flag |= 1;
+  }
+  if (lane == 1) st->inv_norm = nm > 0.0 ? a.inv_nvox / nm : 0.0;
+}
+
+// Equilibrium error from the z pass's per-column residual sums and the convergence decision
+// (equilibrium and stress-constraint errors of iteration it).
+static __device__ __noinline__ void resid_update(const SideArgs& a, double* red) {
+  rows_total<1, 8>(a.partial, a.count, red);
+  if (threadIdx.x != 0) return;
+  IterStatus* st = a.st;
+  const ConvDev& cv = a.conv;
+  const int it = a.it >= 0 ? a.it : st->it_dev;
+  const double sum = ((red[0] + red[1]) + (red[2] + red[3])) + ((red[4] + red[5]) + (red[6] + red[7]));
+  const double e_eq = sqrt(sum) * st->inv_norm, cF = st->cF;
+  const int nan_flag = st->nan_flag | (!isfinite(sum) ? 2 : 0);
+  st->res_sum = sum;
+  st->e_eq = e_eq;
+  st->nan_flag = nan_flag;
+  cv.hist[2 * it] = e_eq;
+  cv.hist[2 * it + 1] = cF;
+  int code = 0;
+  if (nan_flag) code = 2;
+  else if (cv.fixed_iters > 0 ? it + 1 >= cv.fixed_iters : (e_eq < cv.tol && cF < cv.tol)) code = 1;
+  else if (it + 1 >= cv.max_iter) code = 3;
+  if (code) {
+    st->done_it = it;
+    st->done = code;
+  }
+  if (a.it < 0) st->it_dev = it + 1;
+  if (code && a.has_cond) cudaGraphSetConditional(a.cond, 0u);
+}
+
+// True in the CTAs of the extra row, whose first one does the side work.
+__device__ __forceinline__ bool side_row(const SideArgs& a, const Cta& cta, void* smem) {
+  if (a.kind == kSideNone || cta.by != 0) return false;
+  if (cta.bx == 0) {
+    if (a.kind == kSideMean) mean_update(a, static_cast<double*>(smem));
+    else resid_update(a, static_cast<double*>(smem));
+  }
+  return true;
+}
+
 template <typename T>
 struct LineArgs {
   FftDim d;
@@ -531,6 +623,7 @@ struct LineArgs {
   int H, HC, n_o2, NC, hstride;
   const int* done;  // as in XArgs
   long long stride, A, B;
+  SideArgs side;
 };
 
 // Moves a tile between global memory and shared-memory FFT sequences.  Global: n rows of
@@ -590,9 +683,10 @@ __device__ __forceinline__ void line_cta(const LineArgs<T>& a, const Cta& cta) {
   C2<T>* b1 = b0 + (size_t)NC * a.HC * ps;
   const int tid = threadIdx.x, nthr = blockDim.x;
   if (a.done && *a.done) return;
+  if (side_row(a.side, cta, smem_raw)) return;
   const int h0 = (int)cta.bx * a.HC;
   const int hc = min(a.HC, a.H - h0);
-  const int o = (int)cta.by;
+  const int o = (int)cta.by - (a.side.kind != kSideNone ? 1 : 0);
   const size_t base = (size_t)(o / a.n_o2) * a.A + (size_t)(o % a.n_o2) * a.B + (size_t)h0 * a.hstride;
   const int row = hc * NC;  // values per line position, contiguous when hstride == NC
   for (int i = tid; i < n; i += nthr) tw[i] = a.tw[i];
@@ -619,7 +713,7 @@ __device__ __forceinline__ void line_cta(const LineArgs<T>& a, const Cta& cta) {
 }
 
 template <typename T, int SIGN>
-__global__ void __launch_bounds__(kLineThreads) k_line(const LineArgs<T> a) {
+__global__ void __launch_bounds__(kLineThreads) k_line(const __grid_constant__ LineArgs<T> a) {
   line_cta<T, SIGN>(a, own_grid());
 }
 
@@ -641,11 +735,12 @@ __device__ __forceinline__ void line_pencil_cta(const LineArgs<T>& a, const Cta&
   C2<T>* tw = reinterpret_cast<C2<T>*>(smem_raw);
   C2<T>* buf = tw + N;
   if (a.done && *a.done) return;
+  if (side_row(a.side, cta, smem_raw)) return;
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int SP = NC * a.HC;
   const int h0 = (int)cta.bx * a.HC;
   const int S = NC * min(a.HC, a.H - h0);
-  const int o = (int)cta.by;
+  const int o = (int)cta.by - (a.side.kind != kSideNone ? 1 : 0);
   C2<T>* g = a.spec + (size_t)(o / a.n_o2) * a.A + (size_t)(o % a.n_o2) * a.B + (size_t)h0 * NC;
   const size_t gs = (size_t)a.stride;
   const int s = tid % SP, n1 = tid / SP;
@@ -671,7 +766,7 @@ __device__ __forceinline__ void line_pencil_cta(const LineArgs<T>& a, const Cta&
 }
 
 template <typename T, int SIGN, int N1, int N2, int NC>
-__global__ void __launch_bounds__(kPencilThreads) k_line_pencil(const LineArgs<T> a) {
+__global__ void __launch_bounds__(kPencilThreads) k_line_pencil(const __grid_constant__ LineArgs<T> a) {
   line_pencil_cta<T, SIGN, N1, N2, NC>(a, own_grid());
 }
 
@@ -689,15 +784,11 @@ struct ZArgs {
   const T* ky;
   const T* kzt;
   int scheme;   // 0 Willot, 1 Moulinec-Suquet
-  ConvDev conv;
   const int* done;
   T lam0, mu0, invN;
   double* partial;
-  unsigned int* counter;
   IterStatus* st;
-  int it;  // iteration index; < 0: read it from st->it_dev and advance it (graph mode)
-  int has_cond;  // graph mode: clear the loop condition once the increment is decided
-  cudaGraphConditionalHandle cond;
+  int it;  // iteration index; < 0: read it from st->it_dev (graph mode)
 };
 
 constexpr int kZThreads = 256;
@@ -850,7 +941,7 @@ __device__ __forceinline__ void pencil_cols_inplace(C2<T>* b, int ps, int SP, in
 // three barriers between the global load and the global store; twiddles are read through
 // L1.
 template <typename T, int N1, int N2>
-__device__ __forceinline__ void zgreen_cta(const ZArgs<T>& a, const Cta& cta, double (*red)[kNumRed], int& s_last) {
+__device__ __forceinline__ void zgreen_cta(const ZArgs<T>& a, const Cta& cta) {
   constexpr bool kPencil = N1 > 0;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nz = a.nz;
@@ -942,73 +1033,7 @@ __device__ __forceinline__ void zgreen_cta(const ZArgs<T>& a, const Cta& cta, do
       for (int kz = lane; kz < nz; kz += 32) cv += cres[hh * nz + kz];
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) cv += __shfl_xor_sync(0xffffffffu, cv, off);
-      if (lane == 0) {
-        a.partial[(size_t)j * H + h0 + hh] = (double)cv;
-        __threadfence();
-      }
-    }
-  }
-  __syncthreads();
-  if (tid == 0) {
-    __threadfence();
-    const unsigned int prev = atomicAdd(a.counter, 1u);
-    s_last = (prev == cta.count - 1) ? 1 : 0;
-  }
-  __syncthreads();
-  if (s_last) {
-    __threadfence();
-    // the column partials summed in the order of 256 lanes (8 warps) whatever the block
-    // size: lane vl takes b = vl, vl + 256, ... with four accumulators, each warp of lanes
-    // adds by a shuffle tree, then warp 0 adds the 8 warp sums
-    constexpr int kVL = 256;
-    const size_t np = ny * H;
-    const int lane = tid & 31;
-    for (int vl = tid; vl < kVL; vl += nthr) {
-      double q0 = 0.0, q1 = 0.0, q2 = 0.0, q3 = 0.0;
-      size_t b = vl;
-      for (; b + 3 * (size_t)kVL < np; b += 4 * (size_t)kVL) {
-        q0 += __ldcg(&a.partial[b]);
-        q1 += __ldcg(&a.partial[b + kVL]);
-        q2 += __ldcg(&a.partial[b + 2 * (size_t)kVL]);
-        q3 += __ldcg(&a.partial[b + 3 * (size_t)kVL]);
-      }
-      for (; b < np; b += kVL) q0 += __ldcg(&a.partial[b]);
-      double w = (q0 + q1) + (q2 + q3);
-      warp_sum<1>(&w);
-      if (lane == 0) red[vl >> 5][0] = w;
-    }
-    __syncthreads();
-    double v[kNumRed];
-#pragma unroll
-    for (int i = 0; i < kNumRed; ++i) v[i] = 0.0;
-    if (tid < 32) {
-      v[0] = lane < kVL / 32 ? red[lane][0] : 0.0;
-      warp_sum<1>(v);
-    }
-    if (tid == 0) {
-      IterStatus* st = a.st;
-      const double* S = st->sig_mean;
-      const double nrm =
-          fmax(sqrt(S[0] * S[0] + S[1] * S[1] + S[2] * S[2] + 2.0 * (S[3] * S[3] + S[4] * S[4] + S[5] * S[5])),
-               a.conv.s_ref);
-      st->res_sum = v[0];
-      st->e_eq = nrm > 0.0 ? sqrt(v[0]) / ((double)a.nvox * nrm) : 0.0;
-      st->nan_flag |= !isfinite(v[0]) ? 2 : 0;
-      // convergence decision (equilibrium and stress-constraint errors of iteration it)
-      const ConvDev& cv = a.conv;
-      cv.hist[2 * it] = st->e_eq;
-      cv.hist[2 * it + 1] = st->cF;
-      int code = 0;
-      if (st->nan_flag) code = 2;
-      else if (cv.fixed_iters > 0 ? it + 1 >= cv.fixed_iters : (st->e_eq < cv.tol && st->cF < cv.tol)) code = 1;
-      else if (it + 1 >= cv.max_iter) code = 3;
-      if (code) {
-        st->done_it = it;
-        st->done = code;
-      }
-      if (a.it < 0) st->it_dev = it + 1;
-      if (code && a.has_cond) cudaGraphSetConditional(a.cond, 0u);
-      *a.counter = 0u;
+      if (lane == 0) a.partial[(size_t)j * H + h0 + hh] = (double)cv;  // summed by the inverse y pass (resid_update)
     }
   }
 }
@@ -1023,9 +1048,7 @@ struct ZMinBlocks {
 template <typename T, int N1, int N2>
 __global__ void __launch_bounds__(N1 > 0 ? kPencilThreads : kZThreads, ZMinBlocks<T, N1>::value)
     k_zgreen(const ZArgs<T> a) {
-  __shared__ double red[32][kNumRed];
-  __shared__ int s_last;
-  zgreen_cta<T, N1, N2>(a, own_grid(), red, s_last);
+  zgreen_cta<T, N1, N2>(a, own_grid());
 }
 
 // Graph mode: second bound on the device-side iteration loop, independent of the
@@ -1111,18 +1134,16 @@ __global__ void __launch_bounds__(kPencilThreads) k_line_group(const __grid_cons
 
 template <typename T>
 __global__ void __launch_bounds__(kPencilThreads) k_zgreen_group(const __grid_constant__ ZGroup<T> g) {
-  __shared__ double red[32][kNumRed];
-  __shared__ int s_last;
   int m;
   const Cta cta = group_place(g.start, g.gx, g.n, &m);
   const ZArgs<T>& a = g.m[m];
   switch (a.HC <= pencil_max_hc(a.nz) ? a.nz : 0) {
-    case 64: zgreen_cta<T, PencilSplit<64>::N1, PencilSplit<64>::N2>(a, cta, red, s_last); return;
-    case 96: zgreen_cta<T, PencilSplit<96>::N1, PencilSplit<96>::N2>(a, cta, red, s_last); return;
-    case 128: zgreen_cta<T, PencilSplit<128>::N1, PencilSplit<128>::N2>(a, cta, red, s_last); return;
-    case 160: zgreen_cta<T, PencilSplit<160>::N1, PencilSplit<160>::N2>(a, cta, red, s_last); return;
-    case 256: zgreen_cta<T, PencilSplit<256>::N1, PencilSplit<256>::N2>(a, cta, red, s_last); return;
-    default: zgreen_cta<T, 0, 0>(a, cta, red, s_last); return;
+    case 64: zgreen_cta<T, PencilSplit<64>::N1, PencilSplit<64>::N2>(a, cta); return;
+    case 96: zgreen_cta<T, PencilSplit<96>::N1, PencilSplit<96>::N2>(a, cta); return;
+    case 128: zgreen_cta<T, PencilSplit<128>::N1, PencilSplit<128>::N2>(a, cta); return;
+    case 160: zgreen_cta<T, PencilSplit<160>::N1, PencilSplit<160>::N2>(a, cta); return;
+    case 256: zgreen_cta<T, PencilSplit<256>::N1, PencilSplit<256>::N2>(a, cta); return;
+    default: zgreen_cta<T, 0, 0>(a, cta); return;
   }
 }
 
