@@ -624,7 +624,7 @@ rve_status alloc_fields(rve_s* h) {
   // x sequences in shared memory: odd stride nx + 1 for the register transforms of the
   // lengths with a two-step split (conflict-free steps), nx for the Stockham passes
   h->xs = pencil_n1(h->nx) > 0 ? h->nx + 1 : h->nx;
-  h->xsmem = (size_t)(h->nx + 6 * h->L * h->xs) * 2 * sizeof(T);  // FFT buffers; + tables: xsmem_total
+  h->xsmem = (size_t)(h->nx + 2 * xbuf_len(h->L, h->xs)) * 2 * sizeof(T);  // FFT buffers; + tables: xsmem_total
   // y and z passes: tiles of HC kx values x 6 components (two buffers of padded lines);
   // default about 50 KB per CTA so that four CTAs share an SM (the autotuner may change it)
   const size_t tile_budget = 50 * 1024;

@@ -530,6 +530,21 @@ __device__ __forceinline__ pair_t<T> padd(pair_t<T> a, pair_t<T> b) {
   else return pmk<T>(a.x + b.x, a.y + b.y);
 }
 
+// The strain path (e0, de: 12 floats) of a thread in shared memory: read again at every stage
+// instead of being held in registers (volatile, so that the loads stay where they are).  With
+// the rotation and the strain read again after the integration this freed the registers that
+// made the 168-register x pass spill inside the stages: 128^3 743 -> 627 us per launch.  The
+// substep-start kinematic variables in shared memory as well: 650 us.
+__device__ __forceinline__ void load_path(float* v, const float* sc) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(sc) + 48u * threadIdx.x;
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v[4 * i]), "=f"(v[4 * i + 1]), "=f"(v[4 * i + 2]), "=f"(v[4 * i + 3])
+                 : "r"(a + 16u * i));
+}
+__device__ __forceinline__ void load_path(double*, const double*) {}
+
 // Evaluates the rates at elastic strain e0 + s*de - yt.ep and state yt, adds
 // wacc * rates to acc and overwrites yt with y0 + cnext * rates.  FIRST (the first stage of
 // a substep, wacc = 1): the input state is y0 and acc is assigned the rates, so neither the
@@ -546,15 +561,17 @@ __device__ __forceinline__ pair_t<T> padd(pair_t<T> a, pair_t<T> b) {
 // the slip systems' Schmid scale 1/sqrt6 is folded into the moduli (MatDev C*s, the stress
 // itself is not formed), the resolved stresses and the plastic strain rate go through the
 // plane sums (plane_sum, plane_add), and the rate sums are scaled once at the end.
-template <typename T, int NP, bool FIRST = false>
-__device__ __forceinline__ void rk_stage(const MatDev<T>& M, const T* e0, const T* de, T s,
+template <typename T, int NP, bool FIRST = false, bool SC = false>
+__device__ __forceinline__ void rk_stage(const MatDev<T>& M, const T* e0_, const T* de_, T s,
                                          const MPState<T>& y0, MPState<T>& yt, MPState<T>& acc, T wacc,
                                          T cnext, const T* tab) {
   constexpr double kLog2e = 1.44269504088896340736;
   // the stage's input state: y0 in the first stage (so yt needs no copy of it), yt after
   const MPState<T>& yin = FIRST ? y0 : yt;
   // e = e0 + s de - eps_p and the slip-scaled stress ss = C : e / sqrt6 (MatDev's C*s)
-  T e[6], ss[6];
+  T e[6], ss[6], path[12];
+  if constexpr (SC) load_path(path, e0_);
+  const T *e0 = SC ? path : e0_, *de = SC ? path + 6 : de_;
   if constexpr (std::is_same<T, float>::value) {
 #pragma unroll
     for (int c = 0; c < 6; c += 2) {
@@ -1003,15 +1020,22 @@ __device__ __forceinline__ void rk4_fp64(const MatDev<double>& M, const double* 
 // test is a shortcut only: with every rate exactly 0 (inactive systems return 0 in every
 // rate-solve variant) the RK4 substeps leave the state bit for bit unchanged, so results do
 // not depend on it.  Returns false when the test ran and found the increment elastic.
-template <typename T, int NP>
+template <typename T, int NP, bool SC = false>
 __device__ __forceinline__ bool mc_voxel(const MatDev<T>& M, const T* R, const T* eps_n, const T* eps,
-                                         MPState<T>& y, T dt, int nsub, T* sig, const T* tab, bool check = true) {
+                                         MPState<T>& y, T dt, int nsub, T* sig, const T* tab, bool check = true,
+                                         T* sc = nullptr) {
   T e0[6], e1[6], de[6];
   to_crystal<T>(R, eps_n, e0);
   to_crystal<T>(R, eps, e1);
 #pragma unroll
   for (int c = 0; c < 6; ++c) de[c] = e1[c] - e0[c];
   const bool flows = !(check && elastic_increment<T>(M, e0, de, y));
+  if constexpr (SC) {
+    float4* d = reinterpret_cast<float4*>(sc) + 3 * threadIdx.x;
+    d[0] = make_float4(e0[0], e0[1], e0[2], e0[3]);
+    d[1] = make_float4(e0[4], e0[5], de[0], de[1]);
+    d[2] = make_float4(de[2], de[3], de[4], de[5]);
+  }
   if (flows) {
     if constexpr (NP == kDirect && std::is_same<T, double>::value) {
       rk4_fp64(M, e0, de, y, dt, nsub, tab);
@@ -1024,13 +1048,13 @@ __device__ __forceinline__ bool mc_voxel(const MatDev<T>& M, const T* R, const T
       // classical RK4: stages at s0, sh, sh, s1 with weights 1, 2, 2, 1.  The first stage
       // reads y and assigns acc and yt; the other three share one copy of the stage body
       // (not unrolled, which keeps the code compact)
-      rk_stage<T, NP, true>(M, e0, de, s0, y, yt, acc, T(1), T(0.5) * h, tab);
+      rk_stage<T, NP, true, SC>(M, SC ? sc : e0, de, s0, y, yt, acc, T(1), T(0.5) * h, tab);
 #pragma unroll 1
       for (int stg = 1; stg < 4; ++stg) {
         const T s = stg == 3 ? s1 : sh;
         const T wacc = stg == 3 ? T(1) : T(2);
         const T cnext = stg == 1 ? T(0.5) * h : (stg == 2 ? h : T(0));
-        rk_stage<T, NP>(M, e0, de, s, y, yt, acc, wacc, cnext, tab);
+        rk_stage<T, NP, false, SC>(M, SC ? sc : e0, de, s, y, yt, acc, wacc, cnext, tab);
       }
       const T w = h / T(6);
 #pragma unroll
@@ -1041,11 +1065,20 @@ __device__ __forceinline__ bool mc_voxel(const MatDev<T>& M, const T* R, const T
       for (int c = 0; c < 12; ++c) y.al[c] += w * acc.al[c];
     }
   }
-  T ee[6], sc[6];
+  T ee[6], sgc[6];
+  if constexpr (SC) {
+    // the path and (behind the compiler barrier) the rotation are read again
+    asm volatile("" ::: "memory");
+    T path[12];
+    load_path(path, sc);
 #pragma unroll
-  for (int c = 0; c < 6; ++c) ee[c] = e1[c] - y.ep[c];
-  hooke<T>(M, ee, sc);
-  to_sample<T>(R, sc, sig);
+    for (int c = 0; c < 6; ++c) ee[c] = path[c] + path[6 + c] - y.ep[c];
+  } else {
+#pragma unroll
+    for (int c = 0; c < 6; ++c) ee[c] = e1[c] - y.ep[c];
+  }
+  hooke<T>(M, ee, sgc);
+  to_sample<T>(R, sgc, sig);
   return flows;
 }
 
@@ -1068,13 +1101,14 @@ __device__ __forceinline__ void load_voxel(const T* ep, const T* v, const T* al,
   for (int c = 0; c < 12; ++c) y.al[c] = al[c * n + i];
 }
 
-// mc_voxel with the direct tables' out-of-range case: y holds the voxel's state at t_n, which
-// is also at (ep, v, al); the copies keep the arrays of the common path in registers.
+// Integrates a voxel again by the generic solve if its stress is NaN after
+// mc_voxel<T, kDirect> in float (an overstress beyond the tables): its state at t_n is at
+// (ep, v, al), eps_n and eps have the stride n and ne.  The copies keep the arrays of the
+// common path in registers.
 template <typename T, int NP>
-__device__ __forceinline__ bool mc_voxel_any(const MatDev<T>& M, const T* R, const T* eps_n, const T* eps,
-                                             MPState<T>& y, T dt, int nsub, T* sig, const T* tab, bool check,
-                                             const T* ep, const T* v, const T* al, size_t n, size_t i) {
-  const bool flows = mc_voxel<T, NP>(M, R, eps_n, eps, y, dt, nsub, sig, tab, check);
+__device__ __forceinline__ void mc_recover(const MatDev<T>& M, const T* R, const T* eps_n, const T* eps, size_t ne,
+                                           MPState<T>& y, T dt, int nsub, T* sig, const T* ep, const T* v,
+                                           const T* al, size_t n, size_t i) {
   if constexpr (NP == kDirect && std::is_same<T, float>::value) {
     if (sig[0] != sig[0]) {
       T r2[9], a2[6], b2[6], s2[6];
@@ -1084,8 +1118,8 @@ __device__ __forceinline__ bool mc_voxel_any(const MatDev<T>& M, const T* R, con
       for (int c = 0; c < 9; ++c) r2[c] = R[c];
 #pragma unroll
       for (int c = 0; c < 6; ++c) {
-        a2[c] = eps_n[c];
-        b2[c] = eps[c];
+        a2[c] = eps_n[c * n + i];
+        b2[c] = eps[c * ne];
       }
       mc_voxel_generic<T>(M, r2, a2, b2, y2, dt, nsub, s2);
       y = y2;
@@ -1093,7 +1127,6 @@ __device__ __forceinline__ bool mc_voxel_any(const MatDev<T>& M, const T* R, con
       for (int c = 0; c < 6; ++c) sig[c] = s2[c];
     }
   }
-  return flows;
 }
 
 // Starts the copy of the rate tables (16-byte aligned, a multiple of 16 bytes) to shared memory;

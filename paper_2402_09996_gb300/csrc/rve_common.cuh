@@ -40,6 +40,12 @@ __host__ __device__ constexpr int pencil_n1(int n) {
 // most 384 threads, N1 for each of the chunk's 6 HC lines.
 __host__ __device__ constexpr int pencil_max_hc(int n) { return pencil_n1(n) > 0 ? 384 / (6 * pencil_n1(n)) : 0; }
 
+// Complex values of one of the x pass's two FFT buffers: 3 L sequences, at least 12 floats for
+// each of the CTA's 128 threads (kPathInSmem), and even, which keeps both 16-byte aligned.
+__host__ __device__ constexpr int xbuf_len(int L, int xs) {
+  return 3 * L * xs < 768 ? 768 : (3 * L * xs + 1) / 2 * 2;
+}
+
 // One FFT length factored into radix stages (radices 2, 3, 4, 5).
 struct FftDim {
   int n;

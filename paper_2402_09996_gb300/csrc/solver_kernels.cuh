@@ -104,8 +104,8 @@ __device__ __forceinline__ void store_partial(const T* s, double* partial, size_
 
 // Sums of NV rows of n values (row i at p + i n) in an order that does not depend on the block
 // size (a multiple of 32): row i is cut into kSplit contiguous parts, one per virtual warp,
-// whose lane l takes the part's values l, l + 32, ... with four accumulators; a shuffle tree
-// adds the lanes.  A warp instruction of the FP64 pipe takes 64 cycles on its scheduler, so
+// whose lane l takes the part's values l, l + 32, ... with four accumulators and 16 loads in
+// flight; a shuffle tree adds the lanes.  A warp instruction of the FP64 pipe takes 64 cycles on its scheduler, so
 // the rows go to different warps and a tree adds one value.  The NV * kSplit sums are left in
 // red (row i's parts at red[i kSplit ..]); contains a barrier at its end.
 template <int NV, int kSplit>
@@ -115,16 +115,15 @@ __device__ __forceinline__ void rows_total(const double* p, size_t n, double* re
     const size_t part = (n + kSplit - 1) / kSplit, b0 = (w % kSplit) * part;
     const double* r = p + (size_t)(w / kSplit) * n;
     const size_t end = b0 + part < n ? b0 + part : n;
-    double q0 = 0.0, q1 = 0.0, q2 = 0.0, q3 = 0.0;
-    size_t b = b0 + lane;
-    for (; b + 96 < end; b += 128) {
-      q0 += r[b];
-      q1 += r[b + 32];
-      q2 += r[b + 64];
-      q3 += r[b + 96];
+    double q[4] = {0.0, 0.0, 0.0, 0.0};
+    for (size_t b = b0 + lane; b < end; b += 16 * 32) {
+      double x[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) x[j] = b + 32 * j < end ? r[b + 32 * j] : 0.0;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) q[j & 3] += x[j];
     }
-    for (; b < end; b += 32) q0 += r[b];
-    double v = (q0 + q1) + (q2 + q3);
+    double v = (q[0] + q[1]) + (q[2] + q[3]);
     warp_sum<1>(&v);
     if (lane == 0) red[w] = v;
   }
@@ -286,6 +285,11 @@ __device__ __forceinline__ void prefetch_rows(const T* base, int comps, size_t n
   }
 }
 
+// The float update with direct tables keeps each thread's strain path in the FFT buffer that is
+// free between the two transforms.
+template <typename T, int NP>
+constexpr bool kPathInSmem = sizeof(T) == 4 && NP == kDirect;
+
 // One CTA of the x pass (see the file header) at grid place `cta`; k holds a.k or the
 // group's common arguments.  Before the constitutive update a CTA would wait in turn for its
 // spectrum, its tables and its state; the tables' copy to shared memory and the prefetch of
@@ -299,7 +303,7 @@ __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k
   T* tab = reinterpret_cast<T*>(smem_raw);  // rate tables (16-byte rows), then the FFT buffers
   C2<T>* tw = reinterpret_cast<C2<T>*>(tab + table_len<T, NP>(k.M));
   C2<T>* b0 = tw + a.nx;
-  C2<T>* b1 = b0 + 3 * a.L * a.xs;
+  C2<T>* b1 = b0 + xbuf_len(a.L, a.xs);
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int nx = a.nx, H = a.H, half = nx / 2, xs = a.xs;
   const size_t NL = (size_t)a.ny * a.nz;
@@ -403,13 +407,17 @@ __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k
         continue;
       }
     } else {
+      constexpr bool kSC = kPathInSmem<T, NP>;
   #pragma unroll
       for (int c = 0; c < 6; ++c) epsn[c] = a.eps_n[c * nvox + vox];
       MPState<T> y;
       load_voxel<T>(a.ep, a.v, a.al, nvox, vox, y);
-      const uint32_t g = a.grain[vox];
+      const T* Rv = a.Rg + (size_t)a.grain[vox] * 9;
+      if constexpr (!kSC) {
   #pragma unroll
-      for (int i = 0; i < 9; ++i) R[i] = a.Rg[(size_t)g * 9 + i];
+        for (int i = 0; i < 9; ++i) R[i] = Rv[i];
+        Rv = R;
+      }
       // The elastic-increment test saves work only where all 32 voxels of a warp stay
       // elastic; in the developed plastic regime it is wasted.  Iteration 0 of an increment
       // (and the commit) always tests and records per warp whether any voxel flowed;
@@ -417,8 +425,18 @@ __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k
       const size_t grp = ((size_t)line0 * nx + (size_t)(t - (tid & 31))) >> 5;
       const bool record = !COMMIT && a.flow != nullptr && it == 0;
       const bool check = COMMIT || a.flow == nullptr || it == 0 || a.flow[grp] == 0;
-      const bool flowed =
-          mc_voxel_any<T, NP>(k.M, R, epsn, eps, y, k.dt, k.nsub, sig, tab, check, a.ep, a.v, a.al, nvox, vox);
+      const bool flowed = mc_voxel<T, NP, kSC>(k.M, Rv, epsn, eps, y, k.dt, k.nsub, sig, tab, check,
+                                               reinterpret_cast<T*>(oth));
+      if constexpr (kSC) {
+        // the strain is still in the transform's buffer: read it again
+  #pragma unroll
+        for (int p = 0; p < 3; ++p) {
+          const C2<T> z = res[(size_t)(p * nl + l) * xs + x];
+          eps[2 * p] = z.x;
+          eps[2 * p + 1] = z.y;
+        }
+        mc_recover<T, NP>(k.M, Rv, a.eps_n, eps, 1, y, k.dt, k.nsub, sig, a.ep, a.v, a.al, nvox, vox);
+      }
       if (record) {
         const bool any = __any_sync(__activemask(), flowed);
         if ((tid & 31) == 0) a.flow[grp] = any ? 1 : 0;
@@ -1188,7 +1206,8 @@ __global__ void k_material_point(const __grid_constant__ MatDev<T> M, long long 
   }
   MPState<T> y;
   load_voxel<T>(state, state + 6 * n, state + 22 * n, n, (size_t)i, y);
-  mc_voxel_any<T, NP>(M, r, en, e, y, dt, nsub, s, tab, true, state, state + 6 * n, state + 22 * n, n, (size_t)i);
+  mc_voxel<T, NP>(M, r, en, e, y, dt, nsub, s, tab);
+  mc_recover<T, NP>(M, r, eps_n, eps + i, n, y, dt, nsub, s, state, state + 6 * n, state + 22 * n, n, (size_t)i);
 #pragma unroll
   for (int c = 0; c < 6; ++c) state[c * n + i] = y.ep[c];
 #pragma unroll
