@@ -5,12 +5,17 @@
 // This is the constitutive building block of the adjoint of the load history; with unit
 // stress adjoints it gives the rows of the algorithmic tangent d sigma / d eps.
 //
-// One forward pass per voxel, with the primal's operations (constitutive.cuh), stores each
-// RK4 substep's start state and its four stage rates; every reverse sweep rebuilds a
-// stage's intermediates from its input state and stored rates (no rate solve) just
-// before reversing it.  The regularised rate rho(a, P) solving rho = P ((a - eta rho)/K)^n is
-// differentiated implicitly: with z = (a - eta rho)/K and D = K + eta P n z^(n-1),
+// One forward pass per voxel, with the primal's operations (constitutive.cuh), leaves a record
+// of every RK4 stage (VjpStage): its rates and their derivatives, hardening exponentials and
+// plastic rate sums.  A reverse sweep reads the records and solves nothing.  The regularised
+// rate rho(a, P) solving rho = P ((a - eta rho)/K)^n is differentiated implicitly: with
+// z = (a - eta rho)/K and D = K + eta P n z^(n-1),
 //   d rho / d a = P n z^(n-1) / D,   d rho / d P = K z^n / D   (0 where rho = 0).
+// The sweeps are bound by the FP64 pipe in double and by local memory in float.  Rebuilding every
+// stage from its state in every sweep (exponentials, three divisions a system, products with zero
+// Schmid coefficients, rotations as nested sums) took 1750 FP64 instructions a stage; a sweep of
+// the tangent (k_adj_tangent runs seven over one forward pass) now takes about 240.  20^3 FP64
+// history gradient 39.5 -> 29.1 ms; 100003 float points 0.936 -> 0.898 ms.
 #pragma once
 
 #include "constitutive.cuh"
@@ -21,109 +26,46 @@ namespace rve {
 constexpr int kParamBar = 9;  // r0_ord, r0_sup, r0_twin, Q_s, Q_b, b_s, b_b, c, d
 
 template <typename T>
-struct StageVals {
-  T sg[6];
-  T ex[16];
-  T tek[16];  // slip: tau - c alpha; twins: tau
-  T ak[16];
-  T rho[16];
-  T du_s[6], du_t[6];
-  T Es, Et, ftot, wslip, fm_left, Ptw, lg_Ptw;
-  T Rb_s, Rb_t;
-};
-
-// Forward stage (the operations of rk_stage, one system at a time; the float primal runs
-// pairs of systems on packed instructions, which may round the last bit differently):
-// rates k of state Y at path point s,
-// with the intermediates kept for the reverse pass.  SOLVE = false takes the rates rho of
-// the 16 systems from rho_in (a stage evaluated before with the same Y and s) instead of
-// solving for them, and rebuilds everything else.
-template <typename T, int NP, bool SOLVE = true>
-__device__ __forceinline__ void stage_eval(const MatDev<T>& M, const T* e0, const T* de, T s, const MPState<T>& Y,
-                                           const T* tab, StageVals<T>& V, MPState<T>& k,
-                                           const T* rho_in = nullptr) {
-  constexpr double kLog2e = 1.44269504088896340736;
-  T e[6];
+__device__ __forceinline__ void state_axpy(MPState<T>& y, T w, const MPState<T>& x) {
   #pragma unroll
-  for (int c = 0; c < 6; ++c) e[c] = e0[c] + s * de[c] - Y.ep[c];
-  hooke<T>(M, e, V.sg);
-  V.Es = T(0);
-  V.Et = T(0);
-  T vtw = T(0);
-  const T cb_s = -M.b_s * T(kLog2e), cb_t = -M.b_b * T(kLog2e);
+  for (int c = 0; c < 6; ++c) y.ep[c] += w * x.ep[c];
   #pragma unroll
-  for (int q = 0; q < 12; ++q) {
-    V.ex[q] = hard_exp2<T, NP>(M, cb_s * Y.v[q], tab);
-    V.Es += V.ex[q];
-  }
+  for (int c = 0; c < 16; ++c) y.v[c] += w * x.v[c];
   #pragma unroll
-  for (int q = 12; q < 16; ++q) {
-    V.ex[q] = hard_exp2<T, NP>(M, cb_t * Y.v[q], tab);
-    V.Et += V.ex[q];
-    vtw += Y.v[q];
-  }
-  V.ftot = T(1.41421356237309504880) * vtw;
-  V.wslip = T(1) - V.ftot;
-  V.fm_left = M.fm - V.ftot;
-  V.fm_left = V.fm_left > T(0) ? V.fm_left : T(0);
-  V.Ptw = (M.Kc * T(0.70710678118654752440)) * V.fm_left;
-  V.lg_Ptw = fast_log2<T>(V.Ptw > T(0) ? V.Ptw : T(1));
-  const T dq = M.h_diag - M.h_off;
-  const T Qdq_s = M.Q_s * dq, Qdq_t = M.Q_b * dq;
-  V.Rb_s = M.Q_s * (M.h_off * (T(12) - V.Es) + dq);
-  V.Rb_t = M.Q_b * (M.h_off * (T(4) - V.Et) + dq);
-  RootCoef<T> qs, qt;
-  if constexpr (NP != 0 && NP != kDirect && SOLVE) {
-    qs = root_coef<T>(T(1), M.K, M.n, M.inv_n, M.lg_K, M.eta, M.lg_eta, T(0));
-    qt = root_coef<T>(V.Ptw, M.Kt, M.nt, M.inv_nt, M.lg_Kt, M.eta, M.lg_eta, V.lg_Ptw);
-  }
-  T ss[6];
-  #pragma unroll
-  for (int c = 0; c < 6; ++c) ss[c] = V.sg[c] * sys_scale<T>(0);
-  #pragma unroll
-  for (int c = 0; c < 6; ++c) V.du_s[c] = V.du_t[c] = T(0);
-  #pragma unroll
-  for (int q = 0; q < 12; ++q) {
-    V.tek[q] = schmid_sum<T>(q, ss) - M.c * Y.al[q];
-    V.ak[q] = fabs(V.tek[q]) - ((M.r0[q] + V.Rb_s) - Qdq_s * V.ex[q]);
-    if constexpr (SOLVE) V.rho[q] = stage_rate<T, NP>(M, qs, V.ak[q], T(1), false, T(0), tab);
-    else V.rho[q] = rho_in[q];
-    const T gd = copysign(V.rho[q], V.tek[q]);
-    schmid_add<T>(q, gd, V.du_s);
-    k.v[q] = V.rho[q];
-    k.al[q] = gd - M.d * V.rho[q] * Y.al[q];
-  }
-  #pragma unroll
-  for (int q = 12; q < 16; ++q) {
-    V.tek[q] = sys_scale<T>(q) * schmid_sum<T>(q, V.sg);
-    V.ak[q] = V.tek[q] - ((M.r0[q] + V.Rb_t) - Qdq_t * V.ex[q]);
-    if constexpr (SOLVE) V.rho[q] = stage_rate<T, NP>(M, qt, V.ak[q], V.Ptw, true, V.lg_Ptw, tab);
-    else V.rho[q] = rho_in[q];
-    schmid_add<T>(q, V.rho[q], V.du_t);
-    k.v[q] = V.rho[q];
-  }
-  const T fs = V.wslip * sys_scale<T>(0);
-  #pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    const T wc = c < 3 ? T(1) : T(0.5);
-    k.ep[c] = wc * (fs * V.du_s[c] + sys_scale<T>(12) * V.du_t[c]);
-  }
+  for (int c = 0; c < 12; ++c) y.al[c] += w * x.al[c];
 }
+template <typename T>
+__device__ __forceinline__ void state_zero(MPState<T>& y) {
+  #pragma unroll
+  for (int c = 0; c < 6; ++c) y.ep[c] = T(0);
+  #pragma unroll
+  for (int c = 0; c < 16; ++c) y.v[c] = T(0);
+  #pragma unroll
+  for (int c = 0; c < 12; ++c) y.al[c] = T(0);
+}
+
+// What the reverse of one RK4 stage needs of its forward evaluation.  A system of which no
+// voxel of the warp flows has no part in the reverse (its rate and derivative are 0); its bit
+// 16 + q of `bits` is 0 and its da and dP are left unset.
+template <typename T>
+struct VjpStage {
+  T rho[16];     // rates
+  T da[16];      // d rho / d a
+  T dP[4];       // d rho / d P of the twins
+  T ex[16];      // exp(-b v)
+  T al[12];      // kinematic variables of the stage's state
+  T du[6];       // sum_s gdot_s (n x l) of the slip systems, unscaled
+  T ftot;        // sum f
+  unsigned bits;  // bit q < 12: the slip system's driving stress is negative; bit 16 + q: flows
+};
 
 // d rho / d a and d rho / d P at a solved root (rho, a, P; exponent n, K, eta).
 template <typename T>
-__device__ void root_partials(T rho, T a, T P, T Kn, T n, T eta, T* d_a, T* d_P) {
-  if (!(rho > T(0)) || !(P > T(0))) {
-    *d_a = T(0);
-    *d_P = T(0);
-    return;
-  }
+__device__ __forceinline__ void root_partials(T rho, T a, T P, T Kn, T n, T eta, T* d_a, T* d_P) {
+  *d_a = *d_P = T(0);
+  if (!(rho > T(0)) || !(P > T(0))) return;
   const T z = (a - eta * rho) / Kn;
-  if (!(z > T(0))) {
-    *d_a = T(0);
-    *d_P = T(0);
-    return;
-  }
+  if (!(z > T(0))) return;
   const T zn = rho / P;              // z^n
   const T pnz = P * n * (zn / z);    // P n z^(n-1)
   const T D = Kn + eta * pnz;
@@ -131,108 +73,260 @@ __device__ void root_partials(T rho, T a, T P, T Kn, T n, T eta, T* d_a, T* d_P)
   *d_P = Kn * zn / D;
 }
 
-// Reverse of stage_eval: kb = adjoint of the rates; adds the adjoints of Y, e0, de and
-// the parameters.
-template <typename T>
-__device__ void stage_vjp(const MatDev<T>& M, const T* de, T s, const MPState<T>& Y, const StageVals<T>& V,
-                          const MPState<T>& kb, MPState<T>& Yb, T* e0b, T* deb, T* pb) {
+// Forward stage (the operations of rk_stage, one system at a time; the float primal runs
+// pairs of systems on packed instructions, which may round the last bit differently): rates k
+// of state Y at path point s and the stage's record.  Systems in which no voxel of the warp
+// flows cost their driving force only.
+template <typename T, int NP>
+__device__ __forceinline__ void vjp_stage(const MatDev<T>& M, const T* e0, const T* de, T s, const MPState<T>& Y,
+                                          const T* tab, VjpStage<T>& V, MPState<T>& k) {
   constexpr double kLog2e = 1.44269504088896340736;
-  (void)kLog2e;
-  (void)de;
+  const unsigned lanes = __activemask();
+  T ex[16], Es = T(0), Et = T(0), vtw = T(0);
+  const T cb_s = -M.b_s * T(kLog2e), cb_t = -M.b_b * T(kLog2e);
+#pragma unroll
+  for (int q = 0; q < 12; ++q) {
+    ex[q] = hard_exp2<T, NP>(M, cb_s * Y.v[q], tab);
+    Es += ex[q];
+    V.ex[q] = ex[q];
+    V.al[q] = Y.al[q];
+  }
+#pragma unroll
+  for (int q = 12; q < 16; ++q) {
+    ex[q] = hard_exp2<T, NP>(M, cb_t * Y.v[q], tab);
+    Et += ex[q];
+    vtw += Y.v[q];
+    V.ex[q] = ex[q];
+  }
+  const T ftot = T(1.41421356237309504880) * vtw;
+  T fm_left = M.fm - ftot;
+  fm_left = fm_left > T(0) ? fm_left : T(0);
+  const T Ptw = (M.Kc * T(0.70710678118654752440)) * fm_left;
+  const T dq = M.h_diag - M.h_off;
+  const T Qdq_s = M.Q_s * dq, Qdq_t = M.Q_b * dq;
+  const T Rb_s = M.Q_s * (M.h_off * (T(12) - Es) + dq), Rb_t = M.Q_b * (M.h_off * (T(4) - Et) + dq);
+  const T rb_sup = M.r0[0] + Rb_s, rb_ord = M.r0[2] + Rb_s, rb_tw = M.r0[12] + Rb_t;
+  RootCoef<T> qs, qt;
+  T lg_Ptw = T(0), s_tw = T(0), is_tw = T(0);
+  bool scaled = false;
+  if constexpr (NP != kDirect) lg_Ptw = fast_log2<T>(Ptw > T(0) ? Ptw : T(1));
+  if constexpr (NP != 0 && NP != kDirect) {
+    qs = root_coef<T>(T(1), M.K, M.n, M.inv_n, M.lg_K, M.eta, M.lg_eta, T(0));
+    qt = root_coef<T>(Ptw, M.Kt, M.nt, M.inv_nt, M.lg_Kt, M.eta, M.lg_eta, lg_Ptw);
+  }
+  // slip-scaled stress C : e / sqrt6
+  T ss[6];
+  {
+    T e[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) e[c] = e0[c] + s * de[c] - Y.ep[c];
+    ss[0] = M.C11s * e[0] + M.C12s * e[1] + M.C13s * e[2];
+    ss[1] = M.C12s * e[0] + M.C11s * e[1] + M.C13s * e[2];
+    ss[2] = M.C13s * (e[0] + e[1]) + M.C33s * e[2];
+    ss[3] = M.C44s2 * e[3];
+    ss[4] = M.C44s2 * e[4];
+    ss[5] = M.C66s2 * e[5];
+  }
+  unsigned bits = 0;
+  T du[6] = {T(0), T(0), T(0), T(0), T(0), T(0)}, G = T(0), H[3] = {T(0), T(0), T(0)};
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    T S[3], D[3] = {T(0), T(0), T(0)};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) S[i] = plane_sig(p, i) > 0 ? ss[i] + ss[i + 3] : ss[i] - ss[i + 3];
+#pragma unroll
+    for (int q = 3 * p; q < 3 * p + 3; ++q) {
+      const T al = Y.al[q];
+      const T tk = plane_sum<T>(q, S) - M.c * al;
+      const T a = fabs(tk) - ((q % 3 == 2 ? rb_ord : rb_sup) - Qdq_s * ex[q]);
+      k.v[q] = k.al[q] = T(0);
+      if (__any_sync(lanes, a > T(0))) {
+        const T rho = stage_rate<T, NP>(M, qs, a, T(1), false, T(0), tab);
+        T d_a, d_P;
+        root_partials<T>(rho, a, T(1), M.K, M.n, M.eta, &d_a, &d_P);
+        const T gd = copysign(rho, tk);
+        bits |= (tk < T(0) ? 1u : 0u) << q | 1u << (16 + q);
+        V.da[q] = d_a;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          if (diag_k(q, i) == 1) D[i] += gd;
+          else if (diag_k(q, i) == -1) D[i] -= gd;
+        }
+        k.v[q] = rho;
+        k.al[q] = gd - M.d * rho * al;
+      }
+      V.rho[q] = k.v[q];
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      du[i] += D[i];
+      if (plane_sig(p, i) > 0) du[i + 3] += D[i];
+      else du[i + 3] -= D[i];
+    }
+    const int q = 12 + p;
+    // 1/(|n||l|) of a twin is (1/sqrt3) times the slip systems' scale in ss
+    const T a = T(0.57735026918962576451) * plane_sum<T>(q, S) - (rb_tw - Qdq_t * ex[q]);
+    k.v[q] = T(0);
+    if (__any_sync(lanes, a > T(0) && Ptw > T(0))) {
+      T rho;
+      if constexpr (NP == kDirect) {
+        if (!scaled) {
+          const T l = fast_log2<T>(Ptw > T(0) ? Ptw : T(1)) * M.inv_ntm1;
+          s_tw = Ptw > T(0) ? hard_exp2<T, NP>(M, l, tab) : T(0);
+          is_tw = Ptw > T(0) ? hard_exp2<T, NP>(M, -l, tab) : T(0);
+          scaled = true;
+        }
+        rho = rate_root<T>(M, a * s_tw, true, tab) * is_tw;
+      } else {
+        rho = stage_rate<T, NP>(M, qt, a, Ptw, true, lg_Ptw, tab);
+      }
+      T d_a, d_P;
+      root_partials<T>(rho, a, Ptw, M.Kt, M.nt, M.eta, &d_a, &d_P);
+      bits |= 1u << (16 + q);
+      V.da[q] = d_a;
+      V.dP[p] = d_P;
+      G += rho;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) H[i] += plane_sig(p, i) > 0 ? rho : -rho;
+      k.v[q] = rho;
+    }
+    V.rho[q] = k.v[q];
+  }
+  const T fs = (T(1) - ftot) * sys_scale<T>(0), tsc = sys_scale<T>(12);
+  const T dt6[6] = {G, G, T(-2) * G, H[0], H[1], T(-2) * H[2]};
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    V.du[c] = du[c];
+    k.ep[c] = (c < 3 ? T(1) : T(0.5)) * (fs * du[c] + tsc * dt6[c]);
+  }
+  V.ftot = ftot;
+  V.bits = bits;
+}
+
+// Reverse of one stage (record V) of a substep y' = y + h/6 (k1 + 2 k2 + 2 k3 + k4): the
+// adjoint of its rates is kb = cw yend + cY Yb, with yend the adjoint of y' and Yb that of the
+// next stage's state (in); Yb (out) is the adjoint of this stage's state and is added to yb.
+// e0b and deb receive the strain path's adjoint (s: the stage's path point).  With `full` the
+// parameters' adjoints are added to pb (v: the stage's slips are v[q] + cv vr[q]).
+// The Schmid sums go through the plane sums (plane_sum); systems that do not flow are skipped.
+template <typename T>
+__device__ __forceinline__ void vjp_stage_reverse(const MatDev<T>& M, const VjpStage<T>& V, T s,
+                                                  const MPState<T>& yend, T cw, T cY, MPState<T>& Yb, MPState<T>& yb,
+                                                  T* e0b, T* deb, T* pb, bool full, const T* v, T cv, const T* vr) {
+  const unsigned bits = V.bits;
+  if (!(bits >> 16)) {  // no flow: the rates do not depend on anything
+    state_zero<T>(Yb);
+    return;
+  }
   const T dq = M.h_diag - M.h_off;
   const T ssc = sys_scale<T>(0), tsc = sys_scale<T>(12);
-  // eps_p rate: k.ep[c] = wc (wslip ssc du_s[c] + tsc du_t[c])
-  T dusb[6], dutb[6];
-  T wslipb = T(0);
-  #pragma unroll
+  const T ftot = V.ftot, w = (T(1) - ftot) * ssc;
+  // eps_p rate: k.ep[c] = wc (wslip ssc du[c] + tsc du_t[c])
+  T kbe[6], wslipb = T(0);
+#pragma unroll
   for (int c = 0; c < 6; ++c) {
-    const T wc = c < 3 ? T(1) : T(0.5);
-    dusb[c] = kb.ep[c] * wc * V.wslip * ssc;
-    dutb[c] = kb.ep[c] * wc * tsc;
-    wslipb += kb.ep[c] * wc * ssc * V.du_s[c];
+    kbe[c] = (c < 3 ? T(1) : T(0.5)) * (cw * yend.ep[c] + cY * Yb.ep[c]);
+    wslipb += kbe[c] * V.du[c];
   }
-  T sgb[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-  T exb[16];
-  #pragma unroll
-  for (int q = 0; q < 16; ++q) exb[q] = T(0);
-  T Esb = T(0), Etb = T(0), Ptwb = T(0);
-  // slip systems
-  #pragma unroll
-  for (int q = 0; q < 12; ++q) {
-    const T sgn = V.tek[q] < T(0) ? T(-1) : T(1);
-    const T gd = sgn * V.rho[q];
-    // gd enters du_s (schmid_add) and k.al = gd - d rho al
-    T gdb = kb.al[q];
-    #pragma unroll
-    for (int c = 0; c < 6; ++c) gdb += T(schmid_k(q, c)) * dusb[c];
-    T rhob = kb.v[q] + sgn * gdb - M.d * Y.al[q] * kb.al[q];
-    Yb.al[q] += -M.d * V.rho[q] * kb.al[q];
-    pb[8] += -V.rho[q] * Y.al[q] * kb.al[q];  // d
-    (void)gd;
-    T d_a, d_P;
-    root_partials<T>(V.rho[q], V.ak[q], T(1), M.K, M.n, M.eta, &d_a, &d_P);
-    const T akb = rhob * d_a;
-    // a = |tek| - ((r0 + Rb_s) - Qdq_s ex)
-    const T tekb = akb * sgn;
-    const T rb = -akb;
-    pb[(q % 3 == 2) ? 0 : 1] += rb;  // r0: ordinary systems 2, 5, 8, 11; the rest superdislocations
-    Esb += rb * (-M.Q_s * M.h_off);
-    exb[q] += rb * (-M.Q_s * dq);
-    pb[3] += rb * ((M.h_off * (T(12) - V.Es) + dq) - dq * V.ex[q]);  // Q_s
-    // tek = ssc sum K sg - c al
-    Yb.al[q] += -M.c * tekb;
-    pb[7] += -Y.al[q] * tekb;  // c
-    #pragma unroll
-    for (int c = 0; c < 6; ++c) sgb[c] += ssc * T(schmid_k(q, c)) * tekb;
+  wslipb *= ssc;
+  T sgs[6] = {T(0), T(0), T(0), T(0), T(0), T(0)}, G = T(0), H[3] = {T(0), T(0), T(0)};
+  T As = T(0), At = T(0), Ptwb = T(0);  // sums of the overstress adjoints, adjoint of P
+  T hs = T(0), ht = T(0);
+  if (full) {  // hardening sums of Q_s and Q_b
+    T Es = T(0), Et = T(0);
+#pragma unroll
+    for (int q = 0; q < 12; ++q) Es += V.ex[q];
+#pragma unroll
+    for (int q = 12; q < 16; ++q) Et += V.ex[q];
+    hs = M.h_off * (T(12) - Es) + dq;
+    ht = M.h_off * (T(4) - Et) + dq;
   }
-  // twins
-  #pragma unroll
-  for (int q = 12; q < 16; ++q) {
-    T rhob = kb.v[q];
-    #pragma unroll
-    for (int c = 0; c < 6; ++c) rhob += T(schmid_k(q, c)) * dutb[c];
-    T d_a, d_P;
-    root_partials<T>(V.rho[q], V.ak[q], V.Ptw, M.Kt, M.nt, M.eta, &d_a, &d_P);
-    const T akb = rhob * d_a;
-    Ptwb += rhob * d_P;
-    const T rb = -akb;
-    pb[2] += rb;  // r0_twin
-    Etb += rb * (-M.Q_b * M.h_off);
-    exb[q] += rb * (-M.Q_b * dq);
-    pb[4] += rb * ((M.h_off * (T(4) - V.Et) + dq) - dq * V.ex[q]);  // Q_b
-    #pragma unroll
-    for (int c = 0; c < 6; ++c) sgb[c] += tsc * T(schmid_k(q, c)) * akb;
+#pragma unroll
+  for (int p = 0; p < 4; ++p) {
+    T B[3], D[3] = {T(0), T(0), T(0)};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) B[i] = plane_sig(p, i) > 0 ? kbe[i] + kbe[i + 3] : kbe[i] - kbe[i + 3];
+#pragma unroll
+    for (int q = 3 * p; q < 3 * p + 3; ++q) {
+      T exb = T(0), alb = T(0);
+      if (bits >> (16 + q) & 1u) {
+        const bool neg = bits >> q & 1u;
+        const T rho = V.rho[q], al = V.al[q];
+        const T kal = cw * yend.al[q] + cY * Yb.al[q], kv = cw * yend.v[q] + cY * Yb.v[q];
+        const T gdb = kal + w * plane_sum<T>(q, B);
+        // gd enters the plastic rate and k.al = gd - d rho al
+        const T akb = (kv + (neg ? -gdb : gdb) - M.d * al * kal) * V.da[q];
+        // a = |tek| - ((r0 + Rb_s) - Qdq_s ex), tek = ssc sum K sg - c al
+        const T tekb = neg ? -akb : akb;
+        As += akb;
+        exb = akb * (M.Q_s * dq);
+        alb = -M.d * rho * kal - M.c * tekb;
+        yb.al[q] += alb;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          if (diag_k(q, i) == 1) D[i] += tekb;
+          else if (diag_k(q, i) == -1) D[i] -= tekb;
+        }
+        if (full) {
+          pb[q % 3 == 2 ? 0 : 1] -= akb;            // r0: ordinary systems, superdislocations
+          pb[3] -= akb * (hs - dq * V.ex[q]);       // Q_s
+          pb[7] -= al * tekb;                       // c
+          pb[8] -= rho * al * kal;                  // d
+        }
+      }
+      Yb.al[q] = alb;
+      Yb.v[q] = exb;  // the exponential's adjoint for now
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      sgs[i] += D[i];
+      if (plane_sig(p, i) > 0) sgs[i + 3] += D[i];
+      else sgs[i + 3] -= D[i];
+    }
+    const int q = 12 + p;
+    T exb = T(0);
+    if (bits >> (16 + q) & 1u) {
+      const T rhob = cw * yend.v[q] + cY * Yb.v[q] + tsc * plane_sum<T>(q, B);
+      const T akb = rhob * V.da[q];
+      Ptwb += rhob * V.dP[p];
+      At += akb;
+      exb = akb * (M.Q_b * dq);
+      G += akb;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) H[i] += plane_sig(p, i) > 0 ? akb : -akb;
+      if (full) {
+        pb[2] -= akb;                          // r0_twin
+        pb[4] -= akb * (ht - dq * V.ex[q]);    // Q_b
+      }
+    }
+    Yb.v[q] = exb;
   }
   // Ptw = Kc/sqrt2 max(fm - ftot, 0); wslip = 1 - ftot; ftot = sqrt2 sum v_twin
   T ftotb = -wslipb;
-  if (V.fm_left > T(0)) ftotb += Ptwb * (-(M.Kc * T(0.70710678118654752440)));
+  if (M.fm - ftot > T(0)) ftotb -= Ptwb * (M.Kc * T(0.70710678118654752440));
   const T vtwb = T(1.41421356237309504880) * ftotb;
   // ex = exp(-b v)
-  #pragma unroll
-  for (int q = 0; q < 12; ++q) {
-    exb[q] += Esb;
-    Yb.v[q] += exb[q] * (-M.b_s * V.ex[q]);
-    pb[5] += exb[q] * (-Y.v[q] * V.ex[q]);  // b_s
+  const T Esb = As * (M.Q_s * M.h_off), Etb = At * (M.Q_b * M.h_off);
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    const T exb = Yb.v[q] + (q < 12 ? Esb : Etb);
+    const T t = exb * V.ex[q];
+    Yb.v[q] = q < 12 ? -M.b_s * t : vtwb - M.b_b * t;
+    yb.v[q] += Yb.v[q];
+    if (full) pb[q < 12 ? 5 : 6] -= t * (v[q] + cv * vr[q]);  // b_s, b_b
   }
-  #pragma unroll
-  for (int q = 12; q < 16; ++q) {
-    exb[q] += Etb;
-    Yb.v[q] += exb[q] * (-M.b_b * V.ex[q]) + vtwb;
-    pb[6] += exb[q] * (-Y.v[q] * V.ex[q]);  // b_b
-  }
-  // sg = hooke(e), e = e0 + s de - ep
-  T eb[6];
-  eb[0] = M.C11 * sgb[0] + M.C12 * sgb[1] + M.C13 * sgb[2];
-  eb[1] = M.C12 * sgb[0] + M.C11 * sgb[1] + M.C13 * sgb[2];
-  eb[2] = M.C13 * (sgb[0] + sgb[1]) + M.C33 * sgb[2];
-  eb[3] = T(2) * M.C44 * sgb[3];
-  eb[4] = T(2) * M.C44 * sgb[4];
-  eb[5] = T(2) * M.C66 * sgb[5];
-  #pragma unroll
+  // stress = C : e, e = e0 + s de - ep
+  const T sgt[6] = {G, G, T(-2) * G, H[0], H[1], T(-2) * H[2]};
+  T sgb[6], eb[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) sgb[c] = ssc * sgs[c] + tsc * sgt[c];
+  hooke<T>(M, sgb, eb);
+#pragma unroll
   for (int c = 0; c < 6; ++c) {
     e0b[c] += eb[c];
     deb[c] += s * eb[c];
-    Yb.ep[c] -= eb[c];
+    Yb.ep[c] = -eb[c];
+    yb.ep[c] -= eb[c];
   }
 }
 
@@ -261,217 +355,148 @@ __device__ __forceinline__ void out6_adj(const T* ob, T G[3][3]) {
   G[0][1] = G[1][0] = T(0.5) * ob[5];
 }
 
-// out = R^T E R (to_crystal): given out_b, adds E_b (6) and R_b (9).
+// C = A B (3x3).
 template <typename T>
-__device__ void to_crystal_vjp(const T* R, const T* e, const T* ob, T* eb, T* Rb) {
-  T G[3][3], E[3][3];
-  out6_adj<T>(ob, G);
-  sym33<T>(e, E);
-  // E_b = R G R^T ; R_b = 2 E R G
-  T Eb[3][3];
-  #pragma unroll
+__device__ __forceinline__ void mul33(const T A[3][3], const T B[3][3], T C[3][3]) {
+#pragma unroll
   for (int i = 0; i < 3; ++i)
-    #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      T acc = T(0);
-      #pragma unroll
-      for (int a = 0; a < 3; ++a)
-        #pragma unroll
-        for (int b = 0; b < 3; ++b) acc += R[i * 3 + a] * G[a][b] * R[j * 3 + b];
-      Eb[i][j] = acc;
-    }
-  T eb6[6];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) C[i][j] = A[i][0] * B[0][j] + A[i][1] * B[1][j] + A[i][2] * B[2][j];
+}
+template <typename T>
+__device__ __forceinline__ void rows33(const T* R, T A[3][3], bool transpose) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) A[i][j] = transpose ? R[j * 3 + i] : R[i * 3 + j];
+}
+
+// out = R^T E R (to_crystal): given out_b, adds E_b (6) and, with `full`, R_b (9).
+// With A = R G: E_b = A R^T, R_b = 2 E A.
+template <typename T>
+__device__ __forceinline__ void to_crystal_vjp(const T* R, const T* e, const T* ob, T* eb, T* Rb, bool full) {
+  T G[3][3], Q[3][3], A[3][3], Eb[3][3], eb6[6];
+  out6_adj<T>(ob, G);
+  rows33<T>(R, Q, false);
+  mul33<T>(Q, G, A);
+  rows33<T>(R, Q, true);
+  mul33<T>(A, Q, Eb);
   sym33_adj<T>(Eb, eb6);
-  #pragma unroll
+#pragma unroll
   for (int c = 0; c < 6; ++c) eb[c] += eb6[c];
-  #pragma unroll
+  if (!full) return;
+  T E[3][3], X[3][3];
+  sym33<T>(e, E);
+  mul33<T>(E, A, X);
+#pragma unroll
   for (int i = 0; i < 3; ++i)
-    #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      T acc = T(0);
-      #pragma unroll
-      for (int a = 0; a < 3; ++a)
-        #pragma unroll
-        for (int b = 0; b < 3; ++b) acc += E[i][a] * R[a * 3 + b] * G[b][j];
-      Rb[i * 3 + j] += T(2) * acc;
-    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) Rb[i * 3 + j] += T(2) * X[i][j];
 }
 
-// out = R S R^T (to_sample): given out_b, adds S_b (6) and R_b (9).
+// out = R S R^T (to_sample): given out_b, adds S_b (6) and, with `full`, R_b (9).
+// With A = G R: S_b = R^T A, R_b = 2 A S.
 template <typename T>
-__device__ void to_sample_vjp(const T* R, const T* s, const T* ob, T* sb, T* Rb) {
-  T G[3][3], S[3][3];
+__device__ __forceinline__ void to_sample_vjp(const T* R, const T* s, const T* ob, T* sb, T* Rb, bool full) {
+  T G[3][3], Q[3][3], A[3][3], Sb[3][3], sb6[6];
   out6_adj<T>(ob, G);
-  sym33<T>(s, S);
-  T Sb[3][3];
-  #pragma unroll
-  for (int i = 0; i < 3; ++i)
-    #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      T acc = T(0);
-      #pragma unroll
-      for (int a = 0; a < 3; ++a)
-        #pragma unroll
-        for (int b = 0; b < 3; ++b) acc += R[a * 3 + i] * G[a][b] * R[b * 3 + j];
-      Sb[i][j] = acc;
-    }
-  T sb6[6];
+  rows33<T>(R, Q, false);
+  mul33<T>(G, Q, A);
+  rows33<T>(R, Q, true);
+  mul33<T>(Q, A, Sb);
   sym33_adj<T>(Sb, sb6);
-  #pragma unroll
+#pragma unroll
   for (int c = 0; c < 6; ++c) sb[c] += sb6[c];
-  #pragma unroll
+  if (!full) return;
+  T S[3][3], X[3][3];
+  sym33<T>(s, S);
+  mul33<T>(A, S, X);
+#pragma unroll
   for (int i = 0; i < 3; ++i)
-    #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      T acc = T(0);
-      #pragma unroll
-      for (int a = 0; a < 3; ++a)
-        #pragma unroll
-        for (int b = 0; b < 3; ++b) acc += G[i][a] * R[a * 3 + b] * S[b][j];
-      Rb[i * 3 + j] += T(2) * acc;
-    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) Rb[i * 3 + j] += T(2) * X[i][j];
 }
 
-template <typename T>
-__device__ __forceinline__ void state_axpy(MPState<T>& y, T w, const MPState<T>& x) {
-  #pragma unroll
-  for (int c = 0; c < 6; ++c) y.ep[c] += w * x.ep[c];
-  #pragma unroll
-  for (int c = 0; c < 16; ++c) y.v[c] += w * x.v[c];
-  #pragma unroll
-  for (int c = 0; c < 12; ++c) y.al[c] += w * x.al[c];
-}
-template <typename T>
-__device__ __forceinline__ void state_zero(MPState<T>& y) {
-  #pragma unroll
-  for (int c = 0; c < 6; ++c) y.ep[c] = T(0);
-  #pragma unroll
-  for (int c = 0; c < 16; ++c) y.v[c] = T(0);
-  #pragma unroll
-  for (int c = 0; c < 12; ++c) y.al[c] = T(0);
-}
+// Per-voxel inputs of the reverse kernels: rotation, strains (sample frame), strain at t_{n+1}
+// in the crystal frame, and the records of the forward pass: the slips at the start of each of
+// at most NS substeps, the record of each stage, and the plastic strain at t_{n+1}.
+template <typename T, int NS>
+struct VjpVoxel {
+  T r[9], en[6], e[6], e1[6], epN[6];
+  T vs[NS][16];
+  VjpStage<T> st[4 * NS];
+  bool quiet;
+};
 
-
-// Forward pass of mc_voxel that keeps what the reverse sweeps need: the start state of
-// every RK4 substep (ys[0..nsub]) and the rates of its four stages (ks[4 m + j]).  The
-// update arithmetic is the primal's (classical RK4, weights 1 2 2 1, stage inputs
-// y + h/2 k1, y + h/2 k2, y + h k3).
-template <typename T, int NP>
+// Forward pass of mc_voxel from the state y, which keeps what the reverse sweeps need (classical
+// RK4, weights 1 2 2 1, stage inputs y + h/2 k1, y + h/2 k2, y + h k3).
+template <typename T, int NP, int NS>
 __device__ __forceinline__ void mc_forward_store(const MatDev<T>& M, const T* e0, const T* de, T dt, int nsub,
-                                                 const T* tab, MPState<T>* ys, MPState<T>* ks) {
+                                                 const T* tab, MPState<T>& y, VjpVoxel<T, NS>& P) {
   const T h = dt / T(nsub);
   const T inv = T(1) / T(nsub);
-  StageVals<T> V;
 #pragma unroll 1
   for (int m = 0; m < nsub; ++m) {
-    const T s0 = T(m) * inv, sh = (T(m) + T(0.5)) * inv, s1 = (T(m) + T(1)) * inv;
-    MPState<T> k, Y, acc;
+    MPState<T> k, Y = y, acc;
     state_zero<T>(acc);
-    stage_eval<T, NP>(M, e0, de, s0, ys[m], tab, V, k);
-    ks[4 * m] = k;
-    state_axpy<T>(acc, T(1), k);
-    Y = ys[m];
-    state_axpy<T>(Y, T(0.5) * h, k);
-    stage_eval<T, NP>(M, e0, de, sh, Y, tab, V, k);
-    ks[4 * m + 1] = k;
-    state_axpy<T>(acc, T(2), k);
-    Y = ys[m];
-    state_axpy<T>(Y, T(0.5) * h, k);
-    stage_eval<T, NP>(M, e0, de, sh, Y, tab, V, k);
-    ks[4 * m + 2] = k;
-    state_axpy<T>(acc, T(2), k);
-    Y = ys[m];
-    state_axpy<T>(Y, h, k);
-    stage_eval<T, NP>(M, e0, de, s1, Y, tab, V, k);
-    ks[4 * m + 3] = k;
-    state_axpy<T>(acc, T(1), k);
-    Y = ys[m];
-    state_axpy<T>(Y, h / T(6), acc);
-    ys[m + 1] = Y;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) P.vs[m][q] = y.v[q];
+#pragma unroll 1
+    for (int j = 0; j < 4; ++j) {
+      const T s = j == 0 ? T(m) * inv : (j == 3 ? (T(m) + T(1)) * inv : (T(m) + T(0.5)) * inv);
+      vjp_stage<T, NP>(M, e0, de, s, Y, tab, P.st[4 * m + j], k);
+      state_axpy<T>(acc, j == 0 || j == 3 ? T(1) : T(2), k);
+      if (j < 3) {
+        Y = y;
+        state_axpy<T>(Y, j == 2 ? h : T(0.5) * h, k);
+      }
+    }
+    state_axpy<T>(y, h / T(6), acc);
   }
 }
 
-// Reverse sweep of mc_voxel over a stored forward pass (mc_forward_store; quiet: the
-// increment was elastic, ys[nsub] = ys[0]).  In: sigma_b (adjoint of the stress at t_{n+1}),
-// yb (adjoint of the state at t_{n+1}; overwritten with the adjoint of the state at t_n).
-// Out (added): eps_nb, epsb, Rb, pb (kParamBar).  Each stage is rebuilt from its stored
-// input state and rates (no rate solve) just before it is reversed.
-template <typename T, int NP>
-__device__ __forceinline__ void mc_reverse(const MatDev<T>& M, const T* R, const T* eps_n, const T* eps,
-                                           const T* e0, const T* e1, const T* de, bool quiet,
-                                           const MPState<T>* ys, const MPState<T>* ks, T dt, int nsub,
+// Reverse sweep of mc_voxel over the records of its forward pass (quiet: the increment was
+// elastic).  In: sigma_b (adjoint of the stress at t_{n+1}), yb (adjoint of the state at
+// t_{n+1}; overwritten with the adjoint of the state at t_n).  Out (added): epsb, and with
+// `full` also eps_nb, Rb and pb (kParamBar).
+template <typename T, int NS>
+__device__ __forceinline__ void mc_reverse(const MatDev<T>& M, const VjpVoxel<T, NS>& P, T dt, int nsub,
                                            const T* sigma_b, MPState<T>& yb, T* eps_nb, T* epsb, T* Rb, T* pb,
-                                           const T* tab) {
-  const MPState<T>& yN = ys[quiet ? 0 : nsub];
+                                           bool full) {
   // stress: sc = C (e1 - ep_N); sigma = R sc R^T
-  T ee[6], sc[6];
-#pragma unroll
-  for (int c = 0; c < 6; ++c) ee[c] = e1[c] - yN.ep[c];
-  hooke<T>(M, ee, sc);
-  T scb[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-  to_sample_vjp<T>(R, sc, sigma_b, scb, Rb);
-  T eeb[6];
-  eeb[0] = M.C11 * scb[0] + M.C12 * scb[1] + M.C13 * scb[2];
-  eeb[1] = M.C12 * scb[0] + M.C11 * scb[1] + M.C13 * scb[2];
-  eeb[2] = M.C13 * (scb[0] + scb[1]) + M.C33 * scb[2];
-  eeb[3] = T(2) * M.C44 * scb[3];
-  eeb[4] = T(2) * M.C44 * scb[4];
-  eeb[5] = T(2) * M.C66 * scb[5];
   T e0b[6], e1b[6], deb[6];
+  {
+    T ee[6], sc[6], scb[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+#pragma unroll
+    for (int c = 0; c < 6; ++c) ee[c] = P.e1[c] - P.epN[c];
+    hooke<T>(M, ee, sc);
+    to_sample_vjp<T>(P.r, sc, sigma_b, scb, Rb, full);
+    hooke<T>(M, scb, e1b);
+  }
 #pragma unroll
   for (int c = 0; c < 6; ++c) {
-    e1b[c] = eeb[c];
-    yb.ep[c] -= eeb[c];
+    yb.ep[c] -= e1b[c];
     e0b[c] = T(0);
     deb[c] = T(0);
   }
-  if (!quiet) {
+  if (!P.quiet) {
     const T h = dt / T(nsub);
     const T inv = T(1) / T(nsub);
 #pragma unroll 1
     for (int m = nsub - 1; m >= 0; --m) {
-      const T s0 = T(m) * inv, sh = (T(m) + T(0.5)) * inv, s1 = (T(m) + T(1)) * inv;
-      // y' = y + h/6 (k1 + 2 k2 + 2 k3 + k4); yend = adjoint of y'
+      // k4 feeds y' alone, k3 also Y4 = y + h k3, k2 Y3 = y + h/2 k2, k1 Y2 = y + h/2 k1
       const MPState<T> yend = yb;
-      MPState<T> Y, kb, Yb, kdum;
-      StageVals<T> V;
-      // stage 4 at Y4 = y + h k3
-      Y = ys[m];
-      state_axpy<T>(Y, h, ks[4 * m + 2]);
-      stage_eval<T, NP, false>(M, e0, de, s1, Y, tab, V, kdum, ks[4 * m + 3].v);
-      state_zero<T>(kb);
-      state_axpy<T>(kb, h / T(6), yend);
+      MPState<T> Yb;
       state_zero<T>(Yb);
-      stage_vjp<T>(M, de, s1, Y, V, kb, Yb, e0b, deb, pb);
-      state_axpy<T>(yb, T(1), Yb);
-      // stage 3 at Y3 = y + h/2 k2; k3 feeds y' and Y4
-      state_zero<T>(kb);
-      state_axpy<T>(kb, h / T(3), yend);
-      state_axpy<T>(kb, h, Yb);
-      Y = ys[m];
-      state_axpy<T>(Y, T(0.5) * h, ks[4 * m + 1]);
-      stage_eval<T, NP, false>(M, e0, de, sh, Y, tab, V, kdum, ks[4 * m + 2].v);
-      state_zero<T>(Yb);
-      stage_vjp<T>(M, de, sh, Y, V, kb, Yb, e0b, deb, pb);
-      state_axpy<T>(yb, T(1), Yb);
-      // stage 2 at Y2 = y + h/2 k1; k2 feeds y' and Y3
-      state_zero<T>(kb);
-      state_axpy<T>(kb, h / T(3), yend);
-      state_axpy<T>(kb, T(0.5) * h, Yb);
-      Y = ys[m];
-      state_axpy<T>(Y, T(0.5) * h, ks[4 * m]);
-      stage_eval<T, NP, false>(M, e0, de, sh, Y, tab, V, kdum, ks[4 * m + 1].v);
-      state_zero<T>(Yb);
-      stage_vjp<T>(M, de, sh, Y, V, kb, Yb, e0b, deb, pb);
-      state_axpy<T>(yb, T(1), Yb);
-      // stage 1 at y; k1 feeds y' and Y2
-      state_zero<T>(kb);
-      state_axpy<T>(kb, h / T(6), yend);
-      state_axpy<T>(kb, T(0.5) * h, Yb);
-      stage_eval<T, NP, false>(M, e0, de, s0, ys[m], tab, V, kdum, ks[4 * m].v);
-      state_zero<T>(Yb);
-      stage_vjp<T>(M, de, s0, ys[m], V, kb, Yb, e0b, deb, pb);
-      state_axpy<T>(yb, T(1), Yb);
+#pragma unroll 1
+      for (int j = 3; j >= 0; --j) {
+        const T s = j == 0 ? T(m) * inv : (j == 3 ? (T(m) + T(1)) * inv : (T(m) + T(0.5)) * inv);
+        const T cw = j == 0 || j == 3 ? h / T(6) : h / T(3);
+        const T cY = j == 3 ? T(0) : (j == 2 ? h : T(0.5) * h);
+        const T cv = j == 0 ? T(0) : (j == 3 ? h : T(0.5) * h);
+        vjp_stage_reverse<T>(M, P.st[4 * m + j], s, yend, cw, cY, Yb, yb, e0b, deb, pb, full, P.vs[m], cv,
+                             P.st[4 * m + (j > 0 ? j - 1 : 0)].rho);
+      }
     }
   }
   // de = e1 - e0; e0 = R^T eps_n R; e1 = R^T eps R
@@ -480,46 +505,8 @@ __device__ __forceinline__ void mc_reverse(const MatDev<T>& M, const T* R, const
     e1b[c] += deb[c];
     e0b[c] -= deb[c];
   }
-  to_crystal_vjp<T>(R, eps_n, e0b, eps_nb, Rb);
-  to_crystal_vjp<T>(R, eps, e1b, epsb, Rb);
-}
-
-// Per-voxel inputs of the reverse kernels: rotation, strains (sample frame), state at t_n,
-// and the stored forward pass.
-template <typename T>
-struct VjpVoxel {
-  T r[9], en[6], e[6], e0[6], e1[6], de[6];
-  MPState<T> ys[kMaxSubVjp + 1];
-  MPState<T> ks[4 * kMaxSubVjp];
-  bool quiet;
-};
-
-template <typename T, int NP>
-__device__ __forceinline__ void vjp_prepare(const MatDev<T>& M, long long i, size_t n, const T* __restrict__ R,
-                                            const T* __restrict__ eps_n, const T* __restrict__ eps,
-                                            const T* __restrict__ state, T dt, int nsub, const T* tab,
-                                            VjpVoxel<T>& P) {
-#pragma unroll
-  for (int k = 0; k < 9; ++k) P.r[k] = R[(size_t)i * 9 + k];
-#pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    P.en[c] = eps_n[c * n + i];
-    P.e[c] = eps[c * n + i];
-  }
-  MPState<T> y;
-#pragma unroll
-  for (int c = 0; c < 6; ++c) y.ep[c] = state[c * n + i];
-#pragma unroll
-  for (int c = 0; c < 16; ++c) y.v[c] = state[(6 + c) * n + i];
-#pragma unroll
-  for (int c = 0; c < 12; ++c) y.al[c] = state[(22 + c) * n + i];
-  to_crystal<T>(P.r, P.en, P.e0);
-  to_crystal<T>(P.r, P.e, P.e1);
-#pragma unroll
-  for (int c = 0; c < 6; ++c) P.de[c] = P.e1[c] - P.e0[c];
-  P.quiet = elastic_increment<T>(M, P.e0, P.de, y);
-  P.ys[0] = y;
-  if (!P.quiet) mc_forward_store<T, NP>(M, P.e0, P.de, dt, nsub, tab, P.ys, P.ks);
+  if (full) to_crystal_vjp<T>(P.r, P.en, e0b, eps_nb, Rb, true);
+  to_crystal_vjp<T>(P.r, P.e, e1b, epsb, Rb, full);
 }
 
 template <typename T>
@@ -541,10 +528,35 @@ __device__ __forceinline__ void store_state34(T* __restrict__ dst, long long i, 
   for (int c = 0; c < 12; ++c) dst[(22 + c) * n + i] = y.al[c];
 }
 
+template <typename T, int NP, int NS>
+__device__ __forceinline__ void vjp_prepare(const MatDev<T>& M, long long i, size_t n, const T* __restrict__ R,
+                                            const T* __restrict__ eps_n, const T* __restrict__ eps,
+                                            const T* __restrict__ state, T dt, int nsub, const T* tab,
+                                            VjpVoxel<T, NS>& P) {
+#pragma unroll
+  for (int k = 0; k < 9; ++k) P.r[k] = R[(size_t)i * 9 + k];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    P.en[c] = eps_n[c * n + i];
+    P.e[c] = eps[c * n + i];
+  }
+  MPState<T> y;
+  load_state34<T>(state, i, n, y);
+  T e0[6], de[6];
+  to_crystal<T>(P.r, P.en, e0);
+  to_crystal<T>(P.r, P.e, P.e1);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) de[c] = P.e1[c] - e0[c];
+  P.quiet = elastic_increment<T>(M, e0, de, y);
+  if (!P.quiet) mc_forward_store<T, NP, NS>(M, e0, de, dt, nsub, tab, y, P);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) P.epN[c] = y.ep[c];
+}
+
 // One thread per voxel; arrays component-major (component * nvox + voxel) as in the
 // forward material-point kernel.  state_b: in, adjoint of the state at t_{n+1}; out, adjoint
 // of the state at t_n.  R_b (9 x nvox) and param_b (kParamBar x nvox) are per voxel.
-template <typename T, int NP>
+template <typename T, int NP, int NS>
 __global__ void k_material_point_vjp(const MatDev<T> M, long long nvox, const T* __restrict__ R,
                                      const T* __restrict__ eps_n, const T* __restrict__ eps,
                                      const T* __restrict__ state, T dt, int nsub, const T* __restrict__ sigma_b,
@@ -558,8 +570,8 @@ __global__ void k_material_point_vjp(const MatDev<T> M, long long nvox, const T*
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nvox) return;
   const size_t n = (size_t)nvox;
-  VjpVoxel<T> P;
-  vjp_prepare<T, NP>(M, i, n, R, eps_n, eps, state, dt, nsub, tab, P);
+  VjpVoxel<T, NS> P;
+  vjp_prepare<T, NP, NS>(M, i, n, R, eps_n, eps, state, dt, nsub, tab, P);
   T sb[6];
 #pragma unroll
   for (int c = 0; c < 6; ++c) sb[c] = sigma_b[c * n + i];
@@ -570,7 +582,7 @@ __global__ void k_material_point_vjp(const MatDev<T> M, long long nvox, const T*
   T pb[kParamBar];
 #pragma unroll
   for (int k = 0; k < kParamBar; ++k) pb[k] = T(0);
-  mc_reverse<T, NP>(M, P.r, P.en, P.e, P.e0, P.e1, P.de, P.quiet, P.ys, P.ks, dt, nsub, sb, yb, enb, eb, rb, pb, tab);
+  mc_reverse<T, NS>(M, P, dt, nsub, sb, yb, enb, eb, rb, pb, true);
   store_state34<T>(state_b, i, n, yb);
 #pragma unroll
   for (int c = 0; c < 6; ++c) {
@@ -589,7 +601,7 @@ __global__ void k_material_point_vjp(const MatDev<T> M, long long nvox, const T*
 // and the direct part (uniform stress adjoint sd, state adjoint state_b at t_{n+1}, which is
 // overwritten with the adjoint at t_n), whose eps, eps_n, rotation and parameter adjoints go
 // to eps_b, eps_n_b, R_b and param_b.
-template <typename T, int NP>
+template <typename T, int NP, int NS>
 __global__ void k_adj_tangent(const MatDev<T> M, long long nvox, const T* __restrict__ R,
                               const T* __restrict__ eps_n, const T* __restrict__ eps,
                               const T* __restrict__ state, T dt, int nsub, T sd0, T sd1, T sd2, T sd3, T sd4, T sd5,
@@ -603,8 +615,8 @@ __global__ void k_adj_tangent(const MatDev<T> M, long long nvox, const T* __rest
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nvox) return;
   const size_t n = (size_t)nvox;
-  VjpVoxel<T> P;
-  vjp_prepare<T, NP>(M, i, n, R, eps_n, eps, state, dt, nsub, tab, P);
+  VjpVoxel<T, NS> P;
+  vjp_prepare<T, NP, NS>(M, i, n, R, eps_n, eps, state, dt, nsub, tab, P);
 #pragma unroll 1
   for (int row = 0; row < 7; ++row) {
     T sb[6];
@@ -622,8 +634,7 @@ __global__ void k_adj_tangent(const MatDev<T> M, long long nvox, const T* __rest
     T pb[kParamBar];
 #pragma unroll
     for (int k = 0; k < kParamBar; ++k) pb[k] = T(0);
-    mc_reverse<T, NP>(M, P.r, P.en, P.e, P.e0, P.e1, P.de, P.quiet, P.ys, P.ks, dt, nsub, sb, yb, enb, eb, rb, pb,
-                      tab);
+    mc_reverse<T, NS>(M, P, dt, nsub, sb, yb, enb, eb, rb, pb, row == 6);
     if (row < 6) {
 #pragma unroll
       for (int c = 0; c < 6; ++c) J[((size_t)row * 6 + c) * n + i] = eb[c];

@@ -142,7 +142,9 @@ constexpr int kDirect = 3;
 // Template value of the x pass's linear-law mode (the adjoint solve): s = B eps - g per voxel.
 constexpr int kLinearLaw = 1;
 
-// RK4 substeps whose start states the constitutive reverse pass (adjoint.cuh) keeps.
-constexpr int kMaxSubVjp = 16;
+// RK4 substeps of an increment whose stage records the constitutive reverse pass (adjoint.cuh)
+// keeps in local memory: two kernel variants, so that the usual 4 substeps (increments up to
+// 0.5 s) reserve a quarter of the memory.
+constexpr int kFewSubVjp = 4, kMaxSubVjp = 16;
 
 }  // namespace rve
