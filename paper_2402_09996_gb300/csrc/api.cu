@@ -245,7 +245,8 @@ struct rve_s {
   IterStatus* st_host = nullptr;  // pinned
   std::vector<void*> owned;
   // launch geometry
-  int L = 1, xgrid = 0;
+  int L = 1, xgrid = 0, xgrid_most = 0;  // xgrid_most: of any material
+  bool quad = false;  // x pass with four lanes per voxel (XArgs::quad)
   size_t xsmem = 0, ysmem = 0, zsmem = 0;
   int yHC = 1, zHC = 1;
   int xs = 0;  // x-pass shared-memory line stride
@@ -577,8 +578,9 @@ size_t z_smem(const rve_s* h, int hc) {
 // passes: 48^3 FP64 L = 8 2.06 ms (7: 2.78, 5: 2.53, 16: 2.50), 32^3 FP64 L = 4 0.72 (8: 0.86),
 // 20^3 FP64 L = 6 0.41 (7: 0.70), 64^3 FP32 L = 4 141 us (8: 156, 2: 150), 96^3 L = 4 383
 // (5: 401), 128^3 L = 4 804 (3: 824, 5: 815, 2: 863), 160^3 L = 4 1536 (3: 1598, 5: 1596).
-int x_lines_per_cta(int nx, long long NL, int resident) {
-  const long long sms = 152, thr = x_threads();
+// `thr` voxels a round; *rounds: the busiest SM's.
+int x_lines_per_cta(int nx, long long NL, int thr, int resident, long long* rounds) {
+  const long long sms = 152;
   int best = 1;
   long long cost = -1, seq = -1;
   for (int L = 1; L <= NL; ++L) {
@@ -591,7 +593,35 @@ int x_lines_per_cta(int nx, long long NL, int resident) {
       seq = q;
     }
   }
+  *rounds = cost;
   return best;
+}
+
+// Geometry of the x pass.  In double with the direct tables a voxel is updated by four lanes
+// (mc_voxel_quad) where the busiest SM then has no more rounds than with one lane: a round of 32
+// voxels takes about half the time of one of 128.  x pass, increments at 0.3 % strain and above:
+// 16^3 (one round each) 404 -> 216 us; 20^3 (two rounds against one) 415 -> 375 at high strain
+// but 5 % slower at low strain, 24^3 (three against one) 430 -> 600, 32^3 0.86 -> 1.22 ms.
+void x_geometry(rve_s* h) {
+  const bool fp64 = h->opt.precision == RVE_FP64;
+  const size_t elem = fp64 ? sizeof(double) : sizeof(float);
+  long long rounds = 0, rounds4 = 0;
+  h->L = x_lines_per_cta(h->nx, h->NL, x_threads(), fp64 ? 2 : 3, &rounds);
+  h->quad = false;
+  h->xgrid_most = (int)((h->NL + h->L - 1) / h->L);
+  if (fp64) {
+    const int L4 = x_lines_per_cta(h->nx, h->NL, x_threads() / 4, 2, &rounds4);
+    h->xgrid_most = std::max(h->xgrid_most, (int)((h->NL + L4 - 1) / L4));
+    if (variant_of<double>(h->mat) == kDirect && rounds4 <= rounds) {
+      h->quad = true;
+      h->L = L4;
+    }
+  }
+  h->xgrid = (int)((h->NL + h->L - 1) / h->L);
+  // x sequences in shared memory: odd stride nx + 1 for the register transforms of the
+  // lengths with a two-step split (conflict-free steps), nx for the Stockham passes
+  h->xs = pencil_n1(h->nx) > 0 ? h->nx + 1 : h->nx;
+  h->xsmem = (size_t)(h->nx + 2 * xbuf_len(h->L, h->xs)) * 2 * elem;  // FFT buffers; + tables: xsmem_total
 }
 
 template <typename T>
@@ -619,12 +649,7 @@ rve_status alloc_fields(rve_s* h) {
     RVE_CUDA(h, cudaMemsetAsync(h->flow, 0, nflow, h->stream));
   }
   // launch geometry
-  h->L = x_lines_per_cta(h->nx, h->NL, h->opt.precision == RVE_FP64 ? 2 : 3);
-  h->xgrid = (int)((h->NL + h->L - 1) / h->L);
-  // x sequences in shared memory: odd stride nx + 1 for the register transforms of the
-  // lengths with a two-step split (conflict-free steps), nx for the Stockham passes
-  h->xs = pencil_n1(h->nx) > 0 ? h->nx + 1 : h->nx;
-  h->xsmem = (size_t)(h->nx + 2 * xbuf_len(h->L, h->xs)) * 2 * sizeof(T);  // FFT buffers; + tables: xsmem_total
+  x_geometry(h);
   // y and z passes: tiles of HC kx values x 6 components (two buffers of padded lines);
   // default about 50 KB per CTA so that four CTAs share an SM (the autotuner may change it)
   const size_t tile_budget = 50 * 1024;
@@ -640,7 +665,7 @@ rve_status alloc_fields(rve_s* h) {
   h->ysmem = y_smem<T>(h, h->yHC);
   h->zsmem = z_smem<T>(h, h->zHC);
   // x-pass partials per CTA; z-pass partials per (ky, kx) column
-  const size_t npart = std::max((size_t)h->xgrid * kNumRed, (size_t)h->ny * h->H);
+  const size_t npart = std::max((size_t)h->xgrid_most * kNumRed, (size_t)h->ny * h->H);
   if ((s = dalloc(h, (void**)&h->partial, npart * sizeof(double)))) return s;
   if ((s = dalloc(h, (void**)&h->counter, 64))) return s;
   RVE_CUDA(h, cudaMemsetAsync(h->counter, 0, 64, h->stream));
@@ -738,6 +763,7 @@ XArgs<T> x_args(rve_s* h, const void* in, void* out, int it) {
   a.grain = h->grain;
   a.Rg = (const T*)h->Rg;
   a.flow = h->flow;
+  a.quad = h->quad ? 1 : 0;
   a.k.root_tab = (const T*)h->root_tab;
   a.k.M = make_mat<T>(h);
   if (h->lin_mode) {
@@ -1994,6 +2020,7 @@ rve_status rve_set_material(rve_t h, const rve_material* m) {
   h->mat = *m;
   set_reference_medium(h->opt, h->mat, &h->lam0, &h->mu0);
   drop_graphs(h);  // the material is baked into the increment graphs
+  x_geometry(h);
   return h->opt.precision == RVE_FP64 ? upload_root_tab<double>(h) : upload_root_tab<float>(h);
 }
 

@@ -1014,6 +1014,246 @@ __device__ __forceinline__ void rk4_fp64(const MatDev<double>& M, const double* 
   }
 }
 
+// A voxel's update in double by four neighbouring lanes, one slip plane each (its three slip
+// systems and its twin), for grids with fewer warps of voxels than the chip has schedulers: an
+// update is one serial chain of FP64 instructions per warp, and the plane split shortens it (the
+// plastic strain and the stress are formed in all four lanes).  16^3 x pass 404 -> 216 us a
+// launch, increments of 24 iterations 23.9 -> 11.4 ms; x_geometry has the rule.  In plane terms the systems of all planes are alike: with n . l = 0
+// and the signs below, n_i l_i = f (0, 1, -1), (1, 0, -1), (1, -1, 0) and (1, 1, -2).
+struct QuadState {
+  double ep[6], v[4], al[3];
+};
+struct QuadLane {
+  double sig[3];   // plane_sig of the lane's plane
+  double f;        // sign of its first system
+  unsigned mask;   // the voxel's four lanes
+};
+__host__ __device__ constexpr bool quad_sig_minus(int p, int i) { return p == 3 || p == (i == 0 ? 1 : (i == 1 ? 2 : 0)); }
+__host__ __device__ constexpr bool quad_f_minus(int p) { return p == 1 || p == 2; }
+__host__ __device__ constexpr bool quad_planes_hold() {
+  for (int p = 0; p < 4; ++p) {
+    const int f = quad_f_minus(p) ? -1 : 1;
+    const int d[3][3] = {{0, f, -f}, {1, 0, -1}, {1, -1, 0}};
+    for (int i = 0; i < 3; ++i) {
+      if (plane_sig(p, i) != (quad_sig_minus(p, i) ? -1 : 1)) return false;
+      for (int j = 0; j < 3; ++j)
+        if (diag_k(3 * p + j, i) != d[j][i]) return false;
+    }
+  }
+  return true;
+}
+static_assert(quad_planes_hold(), "Table 1 systems: signs of the planes");
+
+__device__ __forceinline__ QuadLane quad_lane() {
+  const int p = threadIdx.x & 3;
+  QuadLane q;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) q.sig[i] = quad_sig_minus(p, i) ? -1.0 : 1.0;
+  q.f = quad_f_minus(p) ? -1.0 : 1.0;
+  q.mask = 0xfu << (threadIdx.x & 28);
+  return q;
+}
+// Sum over the four lanes, the same bits in each.
+__device__ __forceinline__ double quad_sum(unsigned mask, double x) {
+  x += __shfl_xor_sync(mask, x, 1);
+  return x + __shfl_xor_sync(mask, x, 2);
+}
+// Plane sums of the slip-scaled stress at elastic strain e.
+__device__ __forceinline__ void quad_stress(const MatDev<double>& M, const QuadLane& q, const double* e, double* S) {
+  S[0] = M.C11s * e[0] + M.C12s * e[1] + M.C13s * e[2] + q.sig[0] * (M.C44s2 * e[3]);
+  S[1] = M.C12s * e[0] + M.C11s * e[1] + M.C13s * e[2] + q.sig[1] * (M.C44s2 * e[4]);
+  S[2] = M.C13s * (e[0] + e[1]) + M.C33s * e[2] + q.sig[2] * (M.C66s2 * e[5]);
+}
+// Resolved stress of the plane's slip system j.
+__device__ __forceinline__ double quad_resolved(const QuadLane& q, int j, const double* S) {
+  return j == 0 ? q.f * (S[1] - S[2]) : (j == 1 ? S[0] - S[2] : S[0] - S[1]);
+}
+__device__ __forceinline__ double quad_twin(const double* S) {
+  return 0.57735026918962576451 * (S[0] + S[1] - 2.0 * S[2]);
+}
+
+// elastic_increment for the four lanes of a voxel.
+__device__ __forceinline__ bool quad_elastic(const MatDev<double>& M, const QuadLane& q, const double* e0,
+                                             const double* de, const QuadState& y, const double* tab) {
+  constexpr double kLog2e = 1.44269504088896340736;
+  const double* tab_e = tab + (M.rate_len - kExpTab<double>);
+  double ea[6], eb[6], Sa[3], Sb[3], ex[4];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    ea[c] = e0[c] - y.ep[c];
+    eb[c] = e0[c] + de[c] - y.ep[c];
+  }
+  quad_stress(M, q, ea, Sa);
+  quad_stress(M, q, eb, Sb);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) ex[j] = exp2_tab((j < 3 ? -M.b_s : -M.b_b) * kLog2e * y.v[j], tab_e);
+  const double Es = quad_sum(q.mask, ex[0] + ex[1] + ex[2]), Et = quad_sum(q.mask, ex[3]);
+  const double ftot = 1.41421356237309504880 * quad_sum(q.mask, y.v[3]);
+  const double dq = M.h_diag - M.h_off;
+  const double Rb_s = M.Q_s * (M.h_off * (12.0 - Es) + dq), Rb_t = M.Q_b * (M.h_off * (4.0 - Et) + dq);
+  bool quiet = true;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    const double x = M.c * y.al[j], r = (j == 2 ? M.r0[2] : M.r0[0]) + Rb_s - M.Q_s * dq * ex[j];
+    quiet = quiet && !(fabs(quad_resolved(q, j, Sa) - x) - r > 0.0) && !(fabs(quad_resolved(q, j, Sb) - x) - r > 0.0);
+  }
+  if (M.fm - ftot > 0.0) {
+    const double r = M.r0[12] + Rb_t - M.Q_b * dq * ex[3];
+    quiet = quiet && !(quad_twin(Sa) - r > 0.0) && !(quad_twin(Sb) - r > 0.0);
+  }
+  return __all_sync(q.mask, quiet);
+}
+
+// The substeps of rk4_fp64 for the four lanes of a voxel (bit j < 3 of the masks: the lanes' slip
+// systems j, bit 3 the twins).  lanes: the lanes of the warp that call it, whole voxels; the
+// masks are formed over them, so a voxel's lanes take the same exchanges.
+__device__ __forceinline__ void rk4_quad(const MatDev<double>& M, const QuadLane& q, unsigned lanes, const double* e0,
+                                         const double* de, QuadState& y, double dt, int nsub, const double* tab) {
+  constexpr double kLog2e = 1.44269504088896340736;
+  const double* tab_e = tab + (M.rate_len - kExpTab<double>);
+  const double h = dt / (double)nsub, inv = 1.0 / (double)nsub;
+  const double dq = M.h_diag - M.h_off, Qdq_s = M.Q_s * dq, Qdq_t = M.Q_b * dq;
+  QuadState yt = y, acc;
+  double ex[4];
+  double Es = 0.0, Et = 0.0, ftot = 0.0, s_tw = 0.0, is_tw = 0.0;
+  bool scaled = false;
+  unsigned dirty = 0xfu, moved = 0;
+#pragma unroll 1
+  for (int m = 0; m < nsub; ++m) {
+#pragma unroll
+    for (int c = 0; c < 6; ++c) acc.ep[c] = 0.0;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc.v[c] = 0.0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) acc.al[c] = 0.0;
+    unsigned ever = 0;
+#pragma unroll 1
+    for (int stg = 0; stg < 4; ++stg) {
+      const double s = ((double)m + 0.5 * (double)((stg + 1) >> 1)) * inv;
+      const double wacc = stg == 0 || stg == 3 ? 1.0 : 2.0;
+      const double cn = stg == 2 ? h : 0.5 * h;
+      const bool step = stg < 3;
+      if (dirty & 7u) {
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          if (dirty >> j & 1u) ex[j] = exp2_tab(-M.b_s * kLog2e * yt.v[j], tab_e);
+        Es = quad_sum(q.mask, ex[0] + ex[1] + ex[2]);
+      }
+      if (dirty & 8u) {
+        ex[3] = exp2_tab(-M.b_b * kLog2e * yt.v[3], tab_e);
+        Et = quad_sum(q.mask, ex[3]);
+        ftot = 1.41421356237309504880 * quad_sum(q.mask, yt.v[3]);
+        scaled = false;
+      }
+      double fm_left = M.fm - ftot;
+      fm_left = fm_left > 0.0 ? fm_left : 0.0;
+      const double Rb_s = M.Q_s * (M.h_off * (12.0 - Es) + dq), Rb_t = M.Q_b * (M.h_off * (4.0 - Et) + dq);
+      double S[3];
+      {
+        double e[6];
+#pragma unroll
+        for (int c = 0; c < 6; ++c) e[c] = e0[c] + s * de[c] - yt.ep[c];
+        quad_stress(M, q, e, S);
+      }
+      unsigned act = 0;
+      double g[3] = {0.0, 0.0, 0.0}, gt = 0.0;
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const double al = yt.al[j];
+        const double tk = quad_resolved(q, j, S) - M.c * al;
+        const double a = fabs(tk) - ((j == 2 ? M.r0[2] : M.r0[0]) + Rb_s - Qdq_s * ex[j]);
+        if (__any_sync(lanes, a > 0.0)) {
+          const double rho = rate_root<double>(M, a, false, tab);
+          g[j] = copysign(rho, tk);
+          act |= 1u << j;
+          const double ald = g[j] - M.d * rho * al;
+          acc.v[j] += wacc * rho;
+          acc.al[j] += wacc * ald;
+          if (step) {
+            yt.v[j] = y.v[j] + cn * rho;
+            yt.al[j] = y.al[j] + cn * ald;
+          }
+        } else if (step && (moved >> j & 1u)) {
+          yt.v[j] = y.v[j];
+          yt.al[j] = y.al[j];
+        }
+      }
+      const double at = quad_twin(S) - (M.r0[12] + Rb_t - Qdq_t * ex[3]);
+      if (__any_sync(lanes, at > 0.0 && fm_left > 0.0)) {
+        if (!scaled) {
+          const double P = (M.Kc * 0.70710678118654752440) * fm_left;
+          const double l = log2(P > 0.0 ? P : 1.0) * M.inv_ntm1;
+          s_tw = P > 0.0 ? exp2_tab(l, tab_e) : 0.0;
+          is_tw = P > 0.0 ? exp2_tab(-l, tab_e) : 0.0;
+          scaled = true;
+        }
+        gt = rate_root<double>(M, at * s_tw, true, tab) * is_tw;
+        act |= 8u;
+        acc.v[3] += wacc * gt;
+        if (step) yt.v[3] = y.v[3] + cn * gt;
+      } else if (step && (moved & 8u)) {
+        yt.v[3] = y.v[3];
+      }
+      if (act) {
+        // the plane's part x of the normal components of the rate; sig x / 2 that of the shears
+        const double fs = (1.0 - ftot) * sys_scale<double>(0), tg = sys_scale<double>(12) * gt;
+        const double x[3] = {fs * (g[1] + g[2]) + tg, fs * (q.f * g[0] - g[2]) + tg,
+                             fs * (-q.f * g[0] - g[1]) - 2.0 * tg};
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          const double dn = quad_sum(q.mask, x[i]), ds = 0.5 * quad_sum(q.mask, q.sig[i] * x[i]);
+          acc.ep[i] += wacc * dn;
+          acc.ep[i + 3] += wacc * ds;
+          if (step) {
+            yt.ep[i] = y.ep[i] + cn * dn;
+            yt.ep[i + 3] = y.ep[i + 3] + cn * ds;
+          }
+        }
+      } else if (step && moved) {
+#pragma unroll
+        for (int c = 0; c < 6; ++c) yt.ep[c] = y.ep[c];
+      }
+      ever |= act;
+      dirty = step ? act | moved : 0u;
+      if (step) moved = act;
+    }
+    if (ever) {
+      const double w = h / 6.0;
+#pragma unroll
+      for (int c = 0; c < 6; ++c) yt.ep[c] = y.ep[c] = y.ep[c] + w * acc.ep[c];
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        if (ever >> j & 1u) yt.v[j] = y.v[j] = y.v[j] + w * acc.v[j];
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        if (ever >> j & 1u) yt.al[j] = y.al[j] = y.al[j] + w * acc.al[j];
+    }
+    dirty = ever;
+    moved = 0;
+  }
+}
+
+// mc_voxel for the four lanes of a voxel (lanes: the lanes of the warp that call it); the stress
+// is formed in all of them.
+__device__ __forceinline__ void mc_voxel_quad(const MatDev<double>& M, const QuadLane& q, unsigned lanes,
+                                              const double* R,
+                                              const double* eps_n, const double* eps, QuadState& y, double dt,
+                                              int nsub, double* sig, const double* tab) {
+  double e0[6], e1[6], de[6];
+  to_crystal<double>(R, eps_n, e0);
+  to_crystal<double>(R, eps, e1);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) de[c] = e1[c] - e0[c];
+  const bool flows = !quad_elastic(M, q, e0, de, y, tab);
+  const unsigned flowing = __ballot_sync(lanes, flows);
+  if (flows) rk4_quad(M, q, flowing, e0, de, y, dt, nsub, tab);
+  double ee[6], sgc[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) ee[c] = e1[c] - y.ep[c];
+  hooke<double>(M, ee, sgc);
+  to_sample<double>(R, sgc, sig);
+}
+
 // Integrates one voxel over the increment [t_n, t_n + dt] (strain eps_n -> eps, sample
 // frame) and returns the sample-frame stress at t_n + dt; y is updated in place.
 // check: test first whether the increment is elastic and skip the integration if so.  The

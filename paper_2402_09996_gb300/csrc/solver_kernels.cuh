@@ -191,6 +191,7 @@ struct XArgs {
   // some voxel of the group flowed in the increment's first trial iteration, which then
   // skips the elastic-increment test in the later ones (NULL: always test)
   unsigned char* flow;
+  int quad;  // double with the direct tables: four lanes per voxel (xquad_voxels)
 };
 
 // The x transforms of a CTA's nseq packed lines (stride xs >= N + 1 in shared memory) for
@@ -290,6 +291,87 @@ __device__ __forceinline__ void prefetch_rows(const T* base, int comps, size_t n
 template <typename T, int NP>
 constexpr bool kPathInSmem = sizeof(T) == 4 && NP == kDirect;
 
+// The polarisation sigma - C0 : eps of a voxel, packed over its strain in the x sequences.
+template <typename T>
+__device__ __forceinline__ void store_tau(const XCommon<T>& k, const T* sig, const T* eps, C2<T>* seq, size_t stride) {
+  const T tr = k.M.lam0 * (eps[0] + eps[1] + eps[2]);
+  const T m2 = T(2) * k.M.mu0;
+  T tau[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) tau[c] = sig[c] - m2 * eps[c] - (c < 3 ? tr : T(0));
+#pragma unroll
+  for (int p = 0; p < 3; ++p) seq[p * stride] = mk<T>(tau[2 * p], tau[2 * p + 1]);
+}
+
+// The CTA's voxels with four lanes each (mc_voxel_quad): strains from res, polarisations back
+// into it; sums of the stress (sacc) and of the commit's averages (acc) in the lanes.
+template <bool COMMIT>
+__device__ __forceinline__ void xquad_voxels(const XArgs<double>& a, const XCommon<double>& k, C2<double>* res,
+                                             const double* tab, int nl, int line0, double* sacc, double* acc) {
+  const int nx = a.nx, xs = a.xs, g = threadIdx.x & 3;
+  const size_t nvox = (size_t)a.nvox;
+  const unsigned mnx = recip_small((unsigned)nx);
+  const QuadLane q = quad_lane();
+  // the warp's lanes stay together: eight voxels a turn
+  for (int t0 = (int)(threadIdx.x & ~31u) >> 2; t0 < nl * nx; t0 += blockDim.x >> 2) {
+    const int t = t0 + ((int)(threadIdx.x & 31u) >> 2);
+    const unsigned lanes = __ballot_sync(0xffffffffu, t < nl * nx);
+    if (t >= nl * nx) continue;  // the last turn
+    const int l = (int)div_small((unsigned)t, (unsigned)nx, mnx), x = t - l * nx;
+    const size_t vox = ((size_t)line0 + l) * nx + x;
+    double eps[6], epsn[6], sig[6], R[9];
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+      const C2<double> z = res[(size_t)(p * nl + l) * xs + x];
+      eps[2 * p] = z.x;
+      eps[2 * p + 1] = z.y;
+    }
+    QuadState y;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      epsn[c] = a.eps_n[c * nvox + vox];
+      y.ep[c] = a.ep[c * nvox + vox];
+    }
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      y.v[j] = a.v[(3 * g + j) * nvox + vox];
+      y.al[j] = a.al[(3 * g + j) * nvox + vox];
+    }
+    y.v[3] = a.v[(12 + g) * nvox + vox];
+    const double* Rv = a.Rg + (size_t)a.grain[vox] * 9;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) R[i] = Rv[i];
+    mc_voxel_quad(k.M, q, lanes, R, epsn, eps, y, k.dt, k.nsub, sig, tab);
+    __syncwarp(q.mask);  // the voxel's lanes have read its strain and its state
+    if (COMMIT) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        a.v[(3 * g + j) * nvox + vox] = y.v[j];
+        a.al[(3 * g + j) * nvox + vox] = y.al[j];
+        acc[8] += y.v[j];
+      }
+      a.v[(12 + g) * nvox + vox] = y.v[3];
+      acc[7] += 1.41421356237309504880 * y.v[3];
+    }
+    if (g == 0) {
+#pragma unroll
+      for (int c = 0; c < 6; ++c) sacc[c] += sig[c];
+      if (COMMIT) {
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+          a.ep[c * nvox + vox] = y.ep[c];
+          a.eps_n[c * nvox + vox] = eps[c];
+          a.sig_n[c * nvox + vox] = sig[c];
+        }
+        acc[6] += von_mises6<double>(sig);
+      } else {
+        store_tau<double>(k, sig, eps, res + (size_t)l * xs + x, (size_t)nl * xs);
+      }
+    }
+    __syncwarp(lanes);
+  }
+}
+
 // One CTA of the x pass (see the file header) at grid place `cta`; k holds a.k or the
 // group's common arguments.  Before the constitutive update a CTA would wait in turn for its
 // spectrum, its tables and its state; the tables' copy to shared memory and the prefetch of
@@ -379,7 +461,12 @@ __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k
   // the thread's stresses are summed in the field precision over its few voxels (4 at
   // most in float) and added to the FP64 block sum once
   T sacc[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-  for (int t = tid; t < nl * nx; t += nthr) {
+  bool quad = false;
+  if constexpr (std::is_same<T, double>::value && NP == kDirect) {
+    quad = a.quad != 0;
+    if (quad) xquad_voxels<COMMIT>(a, k, res, tab, nl, line0, sacc, acc);
+  }
+  for (int t = quad ? nl * nx : tid; t < nl * nx; t += nthr) {
     const int l = (int)div_small((unsigned)t, (unsigned)nx, mnx), x = t - l * nx;
     const size_t vox = ((size_t)line0 + l) * nx + x;
     T eps[6], epsn[6], sig[6], R[9];
@@ -464,15 +551,7 @@ __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k
         continue;
       }
     }
-    {
-      const T tr = k.M.lam0 * (eps[0] + eps[1] + eps[2]);
-      const T m2 = T(2) * k.M.mu0;
-      T tau[6];
-#pragma unroll
-      for (int c = 0; c < 6; ++c) tau[c] = sig[c] - m2 * eps[c] - (c < 3 ? tr : T(0));
-#pragma unroll
-      for (int p = 0; p < 3; ++p) res[(size_t)(p * nl + l) * xs + x] = mk<T>(tau[2 * p], tau[2 * p + 1]);
-    }
+    store_tau<T>(k, sig, eps, res + (size_t)l * xs + x, (size_t)nl * xs);
   }
   if constexpr (COMMIT || NP == kLinearLaw) {
 #pragma unroll
