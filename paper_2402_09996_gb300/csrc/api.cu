@@ -1846,36 +1846,30 @@ rve_status get_field_t(rve_s* h, int which, int dtype, void* dst, size_t bytes, 
   const size_t n = (size_t)comps * h->nvox;
   const size_t elem = dtype == RVE_DTYPE_F64 ? sizeof(double) : sizeof(float);
   if (!dst || bytes < n * elem) return fail(h, RVE_ERR_INVALID_ARG, "destination too small");
-  // the field in double on the device (in dst itself when it is a device double array),
-  // then narrowed and / or copied to the destination
-  const bool direct = on_dev && dtype == RVE_DTYPE_F64;
-  double* out = (double*)dst;
-  void* tmp = nullptr;
-  void* tmp32 = nullptr;
-  if (!direct) {
-    rve_status s = dalloc(h, &tmp, n * sizeof(double));
-    if (s) return s;
-    out = (double*)tmp;
-  }
-  if (dtype == RVE_DTYPE_F32 && !on_dev) {
-    rve_status s = dalloc(h, &tmp32, n * sizeof(float));
-    if (s) {
-      drop_last(h);
-      return s;
+  // A stored field of the destination's type is copied as it is; any other is written in the
+  // destination's type by one kernel, into dst or, for a host array, a temporary.  (Every copy
+  // went through a temporary in double: 46 components of 256^3 floats moved 24 bytes a value
+  // and allocated up to 2.1 GB a call.)
+  cudaError_t e = cudaSuccess;
+  if (scale == 1.0 && which != RVE_FIELD_VM && elem == sizeof(T)) {
+    e = cudaMemcpyAsync(dst, src, n * elem, on_dev ? cudaMemcpyDefault : cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+  } else {
+    void* out = dst;
+    if (!on_dev) {
+      rve_status s = dalloc(h, &out, n * elem);
+      if (s) return s;
     }
-  }
-  cudaError_t e = which == RVE_FIELD_VM ? launch_von_mises<T>((const T*)src, out, h->nvox, h->stream)
-                                        : launch_to_double<T>((const T*)src, out, (long long)n, h->stream, scale);
-  if (dtype == RVE_DTYPE_F32) {
-    float* f32 = on_dev ? (float*)dst : (float*)tmp32;
-    if (e == cudaSuccess) e = launch_to_float<T>(out, f32, (long long)n, h->stream);
-    if (e == cudaSuccess && !on_dev) e = cudaMemcpyAsync(dst, f32, n * sizeof(float), cudaMemcpyDeviceToHost, h->stream);
-  } else if (e == cudaSuccess && !on_dev) {
-    e = cudaMemcpyAsync(dst, tmp, n * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
-  }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-  for (void* t : {tmp32, tmp}) {  // the last allocations first, as dalloc recorded them
-    if (t) drop_last(h);
+    const T* f = (const T*)src;
+    if (dtype == RVE_DTYPE_F64)
+      e = which == RVE_FIELD_VM ? launch_von_mises<T>(f, (double*)out, h->nvox, h->stream)
+                                : launch_field<T>(f, (double*)out, (long long)n, scale, h->stream);
+    else
+      e = which == RVE_FIELD_VM ? launch_von_mises<T>(f, (float*)out, h->nvox, h->stream)
+                                : launch_field<T>(f, (float*)out, (long long)n, scale, h->stream);
+    if (e == cudaSuccess && !on_dev) e = cudaMemcpyAsync(dst, out, n * elem, cudaMemcpyDeviceToHost, h->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
+    if (!on_dev) drop_last(h);
   }
   if (e != cudaSuccess) return cuda_fail(h, e, "get_fields");
   return RVE_OK;

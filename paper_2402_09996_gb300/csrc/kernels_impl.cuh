@@ -289,51 +289,37 @@ cudaError_t launch_loop_guard(IterStatus* st, int limit, cudaGraphConditionalHan
   return cudaGetLastError();
 }
 
-// dst = scale * src in double (scale 1: an exact widening copy)
-template <typename T>
-__global__ void k_to_double(const T* __restrict__ src, double* __restrict__ dst, long long n, double scale) {
+// dst = scale * src, formed in double and rounded once (scale 1: an exact widening copy or a
+// rounding one).
+template <typename T, typename O>
+__global__ void k_field(const T* __restrict__ src, O* __restrict__ dst, long long n, double scale) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = (double)src[i] * scale;
+  if (i < n) dst[i] = (O)((double)src[i] * scale);
 }
 
-template <typename T>
-cudaError_t launch_to_double(const T* src, double* dst, long long n, cudaStream_t s, double scale) {
+template <typename T, typename O>
+cudaError_t launch_field(const T* src, O* dst, long long n, double scale, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const int thr = 256;
-  k_to_double<T><<<(unsigned)((n + thr - 1) / thr), thr, 0, s>>>(src, dst, n, scale);
+  k_field<T, O><<<(unsigned)((n + thr - 1) / thr), thr, 0, s>>>(src, dst, n, scale);
   return cudaGetLastError();
 }
 
-// double -> float (round to nearest)
-template <typename T>
-__global__ void k_to_float(const double* __restrict__ src, float* __restrict__ dst, long long n) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = (float)src[i];
-}
-
-template <typename T>
-cudaError_t launch_to_float(const double* src, float* dst, long long n, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  const int thr = 256;
-  k_to_float<T><<<(unsigned)((n + thr - 1) / thr), thr, 0, s>>>(src, dst, n);
-  return cudaGetLastError();
-}
-
-template <typename T>
-__global__ void k_von_mises(const T* __restrict__ sig, double* __restrict__ dst, long long nvox) {
+template <typename T, typename O>
+__global__ void k_von_mises(const T* __restrict__ sig, O* __restrict__ dst, long long nvox) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= nvox) return;
   T s[6];
 #pragma unroll
   for (int c = 0; c < 6; ++c) s[c] = sig[c * (size_t)nvox + i];
-  dst[i] = (double)von_mises6<T>(s);
+  dst[i] = (O)von_mises6<T>(s);
 }
 
-template <typename T>
-cudaError_t launch_von_mises(const T* sig6, double* dst, long long nvox, cudaStream_t s) {
+template <typename T, typename O>
+cudaError_t launch_von_mises(const T* sig6, O* dst, long long nvox, cudaStream_t s) {
   if (nvox <= 0) return cudaSuccess;
   const int thr = 256;
-  k_von_mises<T><<<(unsigned)((nvox + thr - 1) / thr), thr, 0, s>>>(sig6, dst, nvox);
+  k_von_mises<T, O><<<(unsigned)((nvox + thr - 1) / thr), thr, 0, s>>>(sig6, dst, nvox);
   return cudaGetLastError();
 }
 
@@ -510,9 +496,10 @@ cudaError_t launch_adj(int which, long long n, cudaStream_t s, const void* p0, c
                                             double, double, cudaStream_t);                                         \
   template cudaError_t launch_shift<T>(C2<T>*, C2<T>*, long long, int, const double*, bool, cudaStream_t);        \
   template cudaError_t launch_xfft<T>(const XFftArgs<T>&, int, dim3, size_t, cudaStream_t);                       \
-  template cudaError_t launch_to_double<T>(const T*, double*, long long, cudaStream_t, double);                   \
-  template cudaError_t launch_to_float<T>(const double*, float*, long long, cudaStream_t);                          \
-  template cudaError_t launch_von_mises<T>(const T*, double*, long long, cudaStream_t);                          \
+  template cudaError_t launch_field<T, double>(const T*, double*, long long, double, cudaStream_t);               \
+  template cudaError_t launch_field<T, float>(const T*, float*, long long, double, cudaStream_t);                 \
+  template cudaError_t launch_von_mises<T, double>(const T*, double*, long long, cudaStream_t);                   \
+  template cudaError_t launch_von_mises<T, float>(const T*, float*, long long, cudaStream_t);                     \
   template cudaError_t launch_loop_guard<T>(IterStatus*, int, cudaGraphConditionalHandle, cudaStream_t);           \
   template cudaError_t launch_adj<T>(int, long long, cudaStream_t, const void*, const void*, const void*, void*,   \
                                      void*, const double*);                                                        \
