@@ -21,6 +21,7 @@
 
 #include "../../include/rve.h"
 #include "launch.h"
+#include "scratch.h"
 #include "solver_kernels.cuh"
 
 using namespace rve;
@@ -725,6 +726,12 @@ std::vector<T> root_tables(const rve_material& m) {
   return std::vector<T>(d.begin(), d.end());
 }
 
+// Room for the rate tables of any material.
+size_t root_tab_bytes(int precision) {
+  return precision == RVE_FP64 ? std::max((size_t)kRootTabs, (size_t)rate_tab_len<double>(true)) * sizeof(double)
+                               : std::max((size_t)kRootTabs, (size_t)rate_tab_len<float>(true)) * sizeof(float);
+}
+
 // The material's rate tables on the device: direct tables are built by a kernel, the Newton
 // variants' start tables on the host.
 template <typename T>
@@ -732,8 +739,7 @@ rve_status upload_root_tab(rve_s* h) {
   const rve_material& m = h->mat;
   const int np = variant_of<T>(m);
   if (!h->root_tab) {
-    // room for any material of the handle
-    rve_status s = dalloc(h, &h->root_tab, std::max((size_t)kRootTabs, (size_t)rate_tab_len<T>(true)) * sizeof(T));
+    rve_status s = dalloc(h, &h->root_tab, root_tab_bytes(h->opt.precision));
     if (s) return s;
   }
   if (np == 0) return RVE_OK;
@@ -2318,12 +2324,15 @@ rve_status rve_material_point(int precision, const rve_material* mat, long long 
   cudaStream_t st = stream ? (cudaStream_t)stream : cudaStreamPerThread;
   tmp.stream = st;
   const int np = precision == RVE_FP64 ? variant_of<double>(*mat) : variant_of<float>(*mat);
-  s = precision == RVE_FP64 ? upload_root_tab<double>(&tmp) : upload_root_tab<float>(&tmp);
-  if (s) {
-    release(&tmp);
-    return fail(nullptr, s, tmp.err);
+  CallScratch tab;
+  cudaError_t e = tab.alloc(root_tab_bytes(precision), st);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return fail(nullptr, RVE_ERR_OOM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   }
-  cudaError_t e;
+  tmp.root_tab = tab.p;
+  s = precision == RVE_FP64 ? upload_root_tab<double>(&tmp) : upload_root_tab<float>(&tmp);
+  if (s) return fail(nullptr, s, tmp.err);
   if (precision == RVE_FP64)
     e = launch_material_point<double>(make_mat<double>(&tmp), np, nvox, (const double*)R, (const double*)eps_n,
                                       (const double*)eps, (double*)state, (double*)sigma, dt, n_sub,
@@ -2333,7 +2342,6 @@ rve_status rve_material_point(int precision, const rve_material* mat, long long 
                                      (const float*)eps, (float*)state, (float*)sigma, (float)dt, n_sub,
                                      (const float*)tmp.root_tab, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  release(&tmp);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "material_point");
   return RVE_OK;
 }
@@ -2355,12 +2363,15 @@ rve_status rve_material_point_vjp(int precision, const rve_material* mat, long l
   cudaStream_t st = stream ? (cudaStream_t)stream : cudaStreamPerThread;
   tmp.stream = st;
   const int np = precision == RVE_FP64 ? variant_of<double>(*mat) : variant_of<float>(*mat);
-  s = precision == RVE_FP64 ? upload_root_tab<double>(&tmp) : upload_root_tab<float>(&tmp);
-  if (s) {
-    release(&tmp);
-    return fail(nullptr, s, tmp.err);
+  CallScratch tab;
+  cudaError_t e = tab.alloc(root_tab_bytes(precision), st);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return fail(nullptr, RVE_ERR_OOM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
   }
-  cudaError_t e;
+  tmp.root_tab = tab.p;
+  s = precision == RVE_FP64 ? upload_root_tab<double>(&tmp) : upload_root_tab<float>(&tmp);
+  if (s) return fail(nullptr, s, tmp.err);
   if (precision == RVE_FP64)
     e = launch_material_point_vjp<double>(make_mat<double>(&tmp), np, nvox, (const double*)R, (const double*)eps_n,
                                           (const double*)eps, (const double*)state, dt, n_sub,
@@ -2373,7 +2384,6 @@ rve_status rve_material_point_vjp(int precision, const rve_material* mat, long l
                                          (const float*)sigma_b, (float*)state_b, (float*)eps_b, (float*)eps_n_b,
                                          (float*)R_b, (float*)param_b, (const float*)tmp.root_tab, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  release(&tmp);
   if (e != cudaSuccess) return cuda_fail(nullptr, e, "material_point_vjp");
   return RVE_OK;
 }

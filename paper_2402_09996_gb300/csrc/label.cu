@@ -22,6 +22,7 @@
 #include <vector>
 
 #include "../../include/rve.h"
+#include "scratch.h"
 
 namespace {
 
@@ -311,13 +312,6 @@ rve_status label_on_device(const char* who, int nx, int ny, int nz, int n_parent
   return RVE_OK;
 }
 
-struct DevBuf {
-  void* p = nullptr;
-  ~DevBuf() {
-    if (p) cudaFree(p);
-  }
-};
-
 }  // namespace
 
 extern "C" rve_status rve_label_voronoi(int nx, int ny, int nz, int n_parent, const double* seeds,
@@ -332,8 +326,9 @@ extern "C" rve_status rve_label_voronoi(int nx, int ny, int nz, int n_parent, co
   // one allocation: 16-byte rows first, then 8-byte, 4-byte and byte arrays; the inputs are
   // packed on the host and copied at once
   const size_t in_bytes = any_twin ? 49 * n : 24 * n, in_room = (49 * n + 15) / 16 * 16;
-  DevBuf buf;
-  LBL_CUDA(cudaMalloc(&buf.p, in_room + (16 + 24 + 32 + 12) * n + (out_on_device ? 0 : nvox * sizeof(uint32_t))));
+  std::vector<char> host(in_bytes);  // outlives the scratch
+  rve::CallScratch buf;
+  LBL_CUDA(buf.alloc(in_room + (16 + 24 + 32 + 12) * n + (out_on_device ? 0 : nvox * sizeof(uint32_t)), st));
   char* d = (char*)buf.p;
   Scratch sc;
   sc.seeds = (double*)d;
@@ -345,7 +340,6 @@ extern "C" rve_status rve_label_voronoi(int nx, int ny, int nz, int n_parent, co
   sc.sums = (unsigned long long*)(d + 40 * n);
   sc.seed_vox = (int*)(d + 72 * n);
   uint32_t* lab = out_on_device ? out : (uint32_t*)(d + 84 * n);
-  std::vector<char> host(in_bytes);
   std::memcpy(host.data(), seeds, 24 * n);
   if (any_twin) {
     std::memcpy(host.data() + 24 * n, twin_normal, 24 * n);
