@@ -600,9 +600,9 @@ int x_lines_per_cta(int nx, long long NL, int thr, int resident, long long* roun
 
 // Geometry of the x pass.  In double with the direct tables a voxel is updated by four lanes
 // (mc_voxel_quad) where the busiest SM then has no more rounds than with one lane: a round of 32
-// voxels takes about half the time of one of 128.  x pass, increments at 0.3 % strain and above:
-// 16^3 (one round each) 404 -> 216 us; 20^3 (two rounds against one) 415 -> 375 at high strain
-// but 5 % slower at low strain, 24^3 (three against one) 430 -> 600, 32^3 0.86 -> 1.22 ms.
+// voxels takes about half the time of one of 128.  Increments of 16 iterations: 16^3 (one round
+// each) 6.9 -> 4.0 ms; 20^3 (two rounds against one) 7.12 -> 6.92 at 0.6 % strain but 6.10 ->
+// 6.37 at 0.2 %; 24^3 (three against one) 7.25 -> 9.91, 32^3 15.2 -> 21.5 ms.
 void x_geometry(rve_s* h) {
   const bool fp64 = h->opt.precision == RVE_FP64;
   const size_t elem = fp64 ? sizeof(double) : sizeof(float);

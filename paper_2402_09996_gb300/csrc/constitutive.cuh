@@ -1017,8 +1017,8 @@ __device__ __forceinline__ void rk4_fp64(const MatDev<double>& M, const double* 
 // A voxel's update in double by four neighbouring lanes, one slip plane each (its three slip
 // systems and its twin), for grids with fewer warps of voxels than the chip has schedulers: an
 // update is one serial chain of FP64 instructions per warp, and the plane split shortens it (the
-// plastic strain and the stress are formed in all four lanes).  16^3 x pass 404 -> 216 us a
-// launch, increments of 24 iterations 23.9 -> 11.4 ms; x_geometry has the rule.  In plane terms the systems of all planes are alike: with n . l = 0
+// plastic strain and the stress are formed in all four lanes).  16^3, increments of 24
+// iterations and 8 substeps: 23.9 -> 11.4 ms; x_geometry has the rule.  In plane terms the systems of all planes are alike: with n . l = 0
 // and the signs below, n_i l_i = f (0, 1, -1), (1, 0, -1), (1, -1, 0) and (1, 1, -2).
 struct QuadState {
   double ep[6], v[4], al[3];
