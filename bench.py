@@ -62,9 +62,8 @@ FLOPS_RHS = 1100                    # one evaluation of the constitutive right-h
 N_SUB = 4                           # RK4 substeps at dt = 0.5 s
 DT = 0.5
 # DRAM bytes (read + write) of one trial x-pass launch on the twinned 128^3 FP32 case, from
-# ncu (dram__bytes_read.sum + dram__bytes_write.sum, mean of three launches in the plastic
-# regime); valid for the x-pass source as profiled, to be re-taken whenever that kernel changes
-XPASS_DRAM_BYTES_128 = 435_345_749
+# ncu (dram__bytes_read.sum + dram__bytes_write.sum, one launch in the plastic regime); valid for the x-pass source as profiled, to be re-taken whenever that kernel changes
+XPASS_DRAM_BYTES_128 = 447_301_376
 
 
 def flops_per_voxit(n_sub):
