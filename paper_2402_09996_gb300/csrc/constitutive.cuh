@@ -98,18 +98,6 @@ __device__ __forceinline__ T schmid_sum(int s, const T* x) {
   return r;
 }
 
-// acc_c += schmid_k(s, c) w
-template <typename T>
-__device__ __forceinline__ void schmid_add(int s, T w, T* acc) {
-#pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    const int k = schmid_k(s, c);
-    if (k == 1) acc[c] += w;
-    else if (k == -1) acc[c] -= w;
-    else if (k != 0) acc[c] += T(k) * w;
-  }
-}
-
 // tau = sigma : m_s = (n . sigma . l) / (|n||l|)
 template <typename T>
 __device__ __forceinline__ T resolved(int s, const T* g) {
