@@ -850,6 +850,15 @@ LineArgs<T> y_args(rve_s* h, void* spec) {
   return a;
 }
 
+// The y pass after the x pass (kSideMean) or after the z pass (kSideResid) of iteration it.
+template <typename T>
+LineArgs<T> y_pass_args(rve_s* h, void* spec, int kind, int it) {
+  LineArgs<T> a = y_args<T>(h, spec);
+  a.side = side_args(h, kind, it);
+  if (kind == kSideResid) a.done = &h->st->stop;
+  return a;
+}
+
 template <typename T>
 ZArgs<T> z_args(rve_s* h, void* spec, const void* Pp, void* Po, int it) {
   ZArgs<T> a{};
@@ -945,8 +954,7 @@ rve_status enqueue_one(rve_s* h, cudaStream_t s, int it, int si, int so, int pi,
   if (timed) tstart(h, 4 * slot + 0, RVE_K_XPASS);
   RVE_CUDA(h, launch_xpass<T>(xa, np, false, h->xgrid, xsmem_total(h), s));
   if (timed) tstop(h, 4 * slot + 0);
-  LineArgs<T> ya = y_args<T>(h, h->spec[so]);
-  ya.side = side_args(h, kSideMean, it);
+  LineArgs<T> ya = y_pass_args<T>(h, h->spec[so], kSideMean, it);
   if (timed) tstart(h, 4 * slot + 1, RVE_K_YFWD);
   RVE_CUDA(h, launch_line<T>(ya, -1, dim3(ygrid_x, h->nz + 1), h->ysmem, s));
   if (timed) tstop(h, 4 * slot + 1);
@@ -954,7 +962,7 @@ rve_status enqueue_one(rve_s* h, cudaStream_t s, int it, int si, int so, int pi,
   if (timed) tstart(h, 4 * slot + 2, RVE_K_ZGREEN);
   RVE_CUDA(h, launch_zgreen<T>(za, dim3(zgrid_x, h->ny), h->zsmem, s));
   if (timed) tstop(h, 4 * slot + 2);
-  ya.side = side_args(h, kSideResid, it);
+  ya = y_pass_args<T>(h, h->spec[so], kSideResid, it);
   if (cond) {
     ya.side.has_cond = 1;
     ya.side.cond = *cond;
@@ -1169,7 +1177,7 @@ rve_status inc_prepare(rve_s* h) {
   // the device-side iteration counters
   for (int c = 0; c < 6; ++c) h->st_host->E[0][c] = h->E_n[c] + h->inc_dE0[c];
   RVE_CUDA(h, cudaMemcpyAsync(h->st->E[0], h->st_host->E[0], 6 * sizeof(double), cudaMemcpyHostToDevice, s));
-  RVE_CUDA(h, cudaMemsetAsync(&h->st->nan_flag, 0, 5 * sizeof(int), s));
+  RVE_CUDA(h, cudaMemsetAsync(&h->st->nan_flag, 0, 6 * sizeof(int), s));
   const Rotation r(h);
   tstart(h, kSlotShift, RVE_K_SHIFT);
   RVE_CUDA(h, launch_shift<T>((C2<T>*)h->spec[r.s0], (C2<T>*)h->backup, h->NL, h->H, h->inc_dE0, false, s));
@@ -1403,10 +1411,8 @@ void group_iter_args(const std::vector<rve_s*>& hs, int which, GroupIter<T>& g) 
     g.x.gx[m] = h->xgrid;
     g.xgrid += h->xgrid;
     g.xsmem = std::max(g.xsmem, xsmem_total(h));
-    g.y.m[m] = y_args<T>(h, h->spec[so]);
-    g.y.m[m].side = side_args(h, kSideMean, -1);
-    g.yi.m[m] = g.y.m[m];
-    g.yi.m[m].side = side_args(h, kSideResid, -1);  // the group guard ends the loop
+    g.y.m[m] = y_pass_args<T>(h, h->spec[so], kSideMean, -1);
+    g.yi.m[m] = y_pass_args<T>(h, h->spec[so], kSideResid, -1);  // the group guard ends the loop
     const int ygx = (h->H + h->yHC - 1) / h->yHC;
     g.y.start[m] = g.yi.start[m] = g.ygrid;
     g.y.gx[m] = g.yi.gx[m] = ygx;
@@ -1731,7 +1737,7 @@ rve_status adjoint_increment(rve_s* h, const double* eps_prev, const double* eps
     RVE_CUDA(h, cudaMemsetAsync(h->P[r.p0], 0, spec_bytes, s));
     std::memset(h->st_host->E[0], 0, sizeof(h->st_host->E[0]));
     RVE_CUDA(h, cudaMemcpyAsync(h->st->E[0], h->st_host->E[0], 6 * sizeof(double), cudaMemcpyHostToDevice, s));
-    RVE_CUDA(h, cudaMemsetAsync(&h->st->nan_flag, 0, 5 * sizeof(int), s));
+    RVE_CUDA(h, cudaMemsetAsync(&h->st->nan_flag, 0, 6 * sizeof(int), s));
     h->lin_mode = true;
     h->lin_sref = g_rms;
     h->lin_B = at(kAdjB);

@@ -99,7 +99,8 @@ struct LoadDev {
   double s_ref;       // floor of the mean-stress norm in the relative errors (0: none)
 };
 
-// Per-iteration device record, written by the last CTA of each reduction.
+// Per-iteration device record, written by the reductions beside the y passes and, for the
+// commit, by its last CTA.
 struct IterStatus {
   double E[2][6];       // E^(i) in slot i%2 (tensor components)
   double sig_mean[6];   // <sigma>^(i)
@@ -113,7 +114,7 @@ struct IterStatus {
   int done_it;          // iteration at which `done` was set
   int it_dev;           // device-driven iteration index (graph mode: advanced by the residual kernel)
   int guard;            // executions of the graph loop body (graph mode)
-  int pad;
+  int stop;             // done as the z pass of the iteration found it (see LineArgs::done)
 };
 
 // Convergence rule evaluated on the device after each iteration's residual.

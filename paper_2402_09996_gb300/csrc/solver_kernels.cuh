@@ -718,7 +718,11 @@ struct LineArgs {
   const C2<T>* tw;
   C2<T>* spec;
   int H, HC, n_o2, NC, hstride;
-  const int* done;  // as in XArgs
+  // nonzero: the pass does nothing.  Not a flag that the pass's own launch writes, or a CTA
+  // (and the warps of one) would go by the time it starts: the inverse pass, beside which
+  // resid_update sets IterStatus::done, goes by `stop`, which the z pass before it copies from
+  // done.  So the iteration that decides an increment transforms its whole spectrum.
+  const int* done;
   long long stride, A, B;
   SideArgs side;
 };
@@ -1048,7 +1052,10 @@ __device__ __forceinline__ void zgreen_cta(const ZArgs<T>& a, const Cta& cta) {
   C2<T>* b1 = b0 + (size_t)6 * a.HC * ps;
   T* cres = reinterpret_cast<T*>((kPencil ? b0 : b1) + (size_t)6 * a.HC * ps);  // HC * nz residual terms
   const int tid = threadIdx.x, nthr = blockDim.x;
-  if (a.done && *a.done) return;
+  if (a.done && *a.done) {
+    if (cta.lin == 0 && tid == 0) a.st->stop = 1;
+    return;
+  }
   const int j = (int)cta.by;
   const int h0 = (int)cta.bx * a.HC;
   const int hc = min(a.HC, a.H - h0);
