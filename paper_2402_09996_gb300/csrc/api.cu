@@ -2027,7 +2027,12 @@ rve_status rve_set_material(rve_t h, const rve_material* m) {
   set_reference_medium(h->opt, h->mat, &h->lam0, &h->mu0);
   drop_graphs(h);  // the material is baked into the increment graphs
   x_geometry(h);
-  return h->opt.precision == RVE_FP64 ? upload_root_tab<double>(h) : upload_root_tab<float>(h);
+  s = h->opt.precision == RVE_FP64 ? upload_root_tab<double>(h) : upload_root_tab<float>(h);
+  if (s) return s;
+  // the per-thread default stream of another thread may run the next step: the tables must
+  // be there for it
+  RVE_CUDA(h, cudaStreamSynchronize(h->stream));
+  return RVE_OK;
 }
 
 rve_status rve_set_mixed_load(rve_t h, const double Edot[6], const uint8_t ctrl[6], const double Sigma[6], double dt) {

@@ -32,3 +32,10 @@ def test_no_pass_goes_by_a_flag_that_its_own_launch_writes(trace, scenario):
     assert {("-1", "1"), ("1", "2")} == {t[:2] for t in lines}
     for sign, _, flag in lines:
         assert flag == ("done" if sign == "-1" else "status")
+
+
+def test_material_tables_are_complete_when_the_call_returns(trace):
+    """The handle's default stream is the calling thread's, so a step from another thread does
+    not wait for work that rve_set_material leaves in flight."""
+    calls = trace("material")
+    assert "rate_table" in calls and calls[-1] == "sync"
