@@ -519,7 +519,9 @@ __device__ __forceinline__ pair_t<T> padd(pair_t<T> a, pair_t<T> b) {
 }
 
 // The strain path (e0, de: 12 floats) of a thread in shared memory: read again at every stage
-// instead of being held in registers (volatile, so that the loads stay where they are).  With
+// instead of being held in registers (volatile, so that the loads stay where they are; they
+// are ordered among each other but not against ordinary stores, so the writer (store_path)
+// puts a compiler barrier on both sides of its stores).  With
 // the rotation and the strain read again after the integration this freed the registers that
 // made the 168-register x pass spill inside the stages: 128^3 743 -> 627 us per launch.  The
 // substep-start kinematic variables in shared memory as well: 650 us.
@@ -532,6 +534,14 @@ __device__ __forceinline__ void load_path(float* v, const float* sc) {
                  : "r"(a + 16u * i));
 }
 __device__ __forceinline__ void load_path(double*, const double*) {}
+__device__ __forceinline__ void store_path(float* sc, const float* e0, const float* de) {
+  float4* d = reinterpret_cast<float4*>(sc) + 3 * threadIdx.x;
+  asm volatile("" ::: "memory");  // after the loads of the thread's voxel before
+  d[0] = make_float4(e0[0], e0[1], e0[2], e0[3]);
+  d[1] = make_float4(e0[4], e0[5], de[0], de[1]);
+  d[2] = make_float4(de[2], de[3], de[4], de[5]);
+  asm volatile("" ::: "memory");  // before the loads of this one
+}
 
 // Evaluates the rates at elastic strain e0 + s*de - yt.ep and state yt, adds
 // wacc * rates to acc and overwrites yt with y0 + cnext * rates.  FIRST (the first stage of
@@ -1258,12 +1268,7 @@ __device__ __forceinline__ bool mc_voxel(const MatDev<T>& M, const T* R, const T
 #pragma unroll
   for (int c = 0; c < 6; ++c) de[c] = e1[c] - e0[c];
   const bool flows = !(check && elastic_increment<T>(M, e0, de, y));
-  if constexpr (SC) {
-    float4* d = reinterpret_cast<float4*>(sc) + 3 * threadIdx.x;
-    d[0] = make_float4(e0[0], e0[1], e0[2], e0[3]);
-    d[1] = make_float4(e0[4], e0[5], de[0], de[1]);
-    d[2] = make_float4(de[2], de[3], de[4], de[5]);
-  }
+  if constexpr (SC) store_path(sc, e0, de);
   if (flows) {
     if constexpr (NP == kDirect && std::is_same<T, double>::value) {
       rk4_fp64(M, e0, de, y, dt, nsub, tab);
