@@ -7,7 +7,8 @@
 //
 // One forward pass per voxel, with the primal's operations (constitutive.cuh), leaves a record
 // of every RK4 stage (VjpStage): its rates and their derivatives, hardening exponentials and
-// plastic rate sums.  A reverse sweep reads the records and solves nothing.  The regularised
+// plastic rate sums (in blocks for more than 8 substeps, see vjp_sweeps).  A reverse sweep reads
+// the records and solves nothing.  The regularised
 // rate rho(a, P) solving rho = P ((a - eta rho)/K)^n is differentiated implicitly: with
 // z = (a - eta rho)/K and D = K + eta P n z^(n-1),
 //   d rho / d a = P n z^(n-1) / D,   d rho / d P = K z^n / D   (0 where rho = 0).
@@ -418,8 +419,8 @@ __device__ __forceinline__ void to_sample_vjp(const T* R, const T* s, const T* o
 }
 
 // Per-voxel inputs of the reverse kernels: rotation, strains (sample frame), strain at t_{n+1}
-// in the crystal frame, and the records of the forward pass: the slips at the start of each of
-// at most NS substeps, the record of each stage, and the plastic strain at t_{n+1}.
+// in the crystal frame, plastic strain at t_{n+1}, and the records of one block of at most NS
+// substeps: the slips at the start of each substep and the record of each stage.
 template <typename T, int NS>
 struct VjpVoxel {
   T r[9], en[6], e[6], e1[6], epN[6];
@@ -428,23 +429,23 @@ struct VjpVoxel {
   bool quiet;
 };
 
-// Forward pass of mc_voxel from the state y, which keeps what the reverse sweeps need (classical
-// RK4, weights 1 2 2 1, stage inputs y + h/2 k1, y + h/2 k2, y + h k3).
+// Substeps m0 .. m1 - 1 of mc_voxel from the state y (classical RK4, weights 1 2 2 1, stage inputs
+// y + h/2 k1, y + h/2 k2, y + h k3), which leave the records that the reverse sweeps need.
 template <typename T, int NP, int NS>
-__device__ __forceinline__ void mc_forward_store(const MatDev<T>& M, const T* e0, const T* de, T dt, int nsub,
-                                                 const T* tab, MPState<T>& y, VjpVoxel<T, NS>& P) {
+__device__ __forceinline__ void mc_forward_store(const MatDev<T>& M, const T* e0, const T* de, T dt, int nsub, int m0,
+                                                 int m1, const T* tab, MPState<T>& y, VjpVoxel<T, NS>& P) {
   const T h = dt / T(nsub);
   const T inv = T(1) / T(nsub);
 #pragma unroll 1
-  for (int m = 0; m < nsub; ++m) {
+  for (int m = m0; m < m1; ++m) {
     MPState<T> k, Y = y, acc;
     state_zero<T>(acc);
 #pragma unroll
-    for (int q = 0; q < 16; ++q) P.vs[m][q] = y.v[q];
+    for (int q = 0; q < 16; ++q) P.vs[m - m0][q] = y.v[q];
 #pragma unroll 1
     for (int j = 0; j < 4; ++j) {
       const T s = j == 0 ? T(m) * inv : (j == 3 ? (T(m) + T(1)) * inv : (T(m) + T(0.5)) * inv);
-      vjp_stage<T, NP>(M, e0, de, s, Y, tab, P.st[4 * m + j], k);
+      vjp_stage<T, NP>(M, e0, de, s, Y, tab, P.st[4 * (m - m0) + j], k);
       state_axpy<T>(acc, j == 0 || j == 3 ? T(1) : T(2), k);
       if (j < 3) {
         Y = y;
@@ -455,58 +456,70 @@ __device__ __forceinline__ void mc_forward_store(const MatDev<T>& M, const T* e0
   }
 }
 
-// Reverse sweep of mc_voxel over the records of its forward pass (quiet: the increment was
-// elastic).  In: sigma_b (adjoint of the stress at t_{n+1}), yb (adjoint of the state at
-// t_{n+1}; overwritten with the adjoint of the state at t_n).  Out (added): epsb, and with
-// `full` also eps_nb, Rb and pb (kParamBar).
+// A reverse sweep of mc_voxel over the records of its forward pass: the state adjoint yb (at
+// t_{n+1}, at the end of the sweep at t_n) and the adjoints of the strain path (crystal frame:
+// e0, its step and e1).
+template <typename T>
+struct VjpSeed {
+  MPState<T> yb;
+  T e0b[6], deb[6], e1b[6];
+};
+
+// Start of a sweep: the stress sigma = R sc R^T, sc = C (e1 - ep_N), with adjoint sigma_b.
 template <typename T, int NS>
-__device__ __forceinline__ void mc_reverse(const MatDev<T>& M, const VjpVoxel<T, NS>& P, T dt, int nsub,
-                                           const T* sigma_b, MPState<T>& yb, T* eps_nb, T* epsb, T* Rb, T* pb,
-                                           bool full) {
-  // stress: sc = C (e1 - ep_N); sigma = R sc R^T
-  T e0b[6], e1b[6], deb[6];
-  {
-    T ee[6], sc[6], scb[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+__device__ __forceinline__ void reverse_stress(const MatDev<T>& M, const VjpVoxel<T, NS>& P, const T* sigma_b,
+                                               VjpSeed<T>& S, T* Rb, bool full) {
+  T ee[6], sc[6], scb[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
 #pragma unroll
-    for (int c = 0; c < 6; ++c) ee[c] = P.e1[c] - P.epN[c];
-    hooke<T>(M, ee, sc);
-    to_sample_vjp<T>(P.r, sc, sigma_b, scb, Rb, full);
-    hooke<T>(M, scb, e1b);
-  }
+  for (int c = 0; c < 6; ++c) ee[c] = P.e1[c] - P.epN[c];
+  hooke<T>(M, ee, sc);
+  to_sample_vjp<T>(P.r, sc, sigma_b, scb, Rb, full);
+  hooke<T>(M, scb, S.e1b);
 #pragma unroll
   for (int c = 0; c < 6; ++c) {
-    yb.ep[c] -= e1b[c];
-    e0b[c] = T(0);
-    deb[c] = T(0);
+    S.yb.ep[c] -= S.e1b[c];
+    S.e0b[c] = T(0);
+    S.deb[c] = T(0);
   }
-  if (!P.quiet) {
-    const T h = dt / T(nsub);
-    const T inv = T(1) / T(nsub);
+}
+
+// The substeps m0 .. m1 - 1, whose records are in P; with `full` also pb (kParamBar, added).
+template <typename T, int NS>
+__device__ __forceinline__ void reverse_substeps(const MatDev<T>& M, const VjpVoxel<T, NS>& P, T dt, int nsub, int m0,
+                                                 int m1, VjpSeed<T>& S, T* pb, bool full) {
+  const T h = dt / T(nsub);
+  const T inv = T(1) / T(nsub);
 #pragma unroll 1
-    for (int m = nsub - 1; m >= 0; --m) {
-      // k4 feeds y' alone, k3 also Y4 = y + h k3, k2 Y3 = y + h/2 k2, k1 Y2 = y + h/2 k1
-      const MPState<T> yend = yb;
-      MPState<T> Yb;
-      state_zero<T>(Yb);
+  for (int m = m1 - 1; m >= m0; --m) {
+    // k4 feeds y' alone, k3 also Y4 = y + h k3, k2 Y3 = y + h/2 k2, k1 Y2 = y + h/2 k1
+    const MPState<T> yend = S.yb;
+    MPState<T> Yb;
+    state_zero<T>(Yb);
+    const VjpStage<T>* st = &P.st[4 * (m - m0)];
 #pragma unroll 1
-      for (int j = 3; j >= 0; --j) {
-        const T s = j == 0 ? T(m) * inv : (j == 3 ? (T(m) + T(1)) * inv : (T(m) + T(0.5)) * inv);
-        const T cw = j == 0 || j == 3 ? h / T(6) : h / T(3);
-        const T cY = j == 3 ? T(0) : (j == 2 ? h : T(0.5) * h);
-        const T cv = j == 0 ? T(0) : (j == 3 ? h : T(0.5) * h);
-        vjp_stage_reverse<T>(M, P.st[4 * m + j], s, yend, cw, cY, Yb, yb, e0b, deb, pb, full, P.vs[m], cv,
-                             P.st[4 * m + (j > 0 ? j - 1 : 0)].rho);
-      }
+    for (int j = 3; j >= 0; --j) {
+      const T s = j == 0 ? T(m) * inv : (j == 3 ? (T(m) + T(1)) * inv : (T(m) + T(0.5)) * inv);
+      const T cw = j == 0 || j == 3 ? h / T(6) : h / T(3);
+      const T cY = j == 3 ? T(0) : (j == 2 ? h : T(0.5) * h);
+      const T cv = j == 0 ? T(0) : (j == 3 ? h : T(0.5) * h);
+      vjp_stage_reverse<T>(M, st[j], s, yend, cw, cY, Yb, S.yb, S.e0b, S.deb, pb, full, P.vs[m - m0], cv,
+                           st[j > 0 ? j - 1 : 0].rho);
     }
   }
-  // de = e1 - e0; e0 = R^T eps_n R; e1 = R^T eps R
+}
+
+// End of a sweep: de = e1 - e0; e0 = R^T eps_n R; e1 = R^T eps R.  Adds to epsb and, with `full`,
+// to eps_nb and Rb.
+template <typename T, int NS>
+__device__ __forceinline__ void reverse_strains(const VjpVoxel<T, NS>& P, VjpSeed<T>& S, T* eps_nb, T* epsb, T* Rb,
+                                                bool full) {
 #pragma unroll
   for (int c = 0; c < 6; ++c) {
-    e1b[c] += deb[c];
-    e0b[c] -= deb[c];
+    S.e1b[c] += S.deb[c];
+    S.e0b[c] -= S.deb[c];
   }
-  if (full) to_crystal_vjp<T>(P.r, P.en, e0b, eps_nb, Rb, true);
-  to_crystal_vjp<T>(P.r, P.e, e1b, epsb, Rb, full);
+  if (full) to_crystal_vjp<T>(P.r, P.en, S.e0b, eps_nb, Rb, true);
+  to_crystal_vjp<T>(P.r, P.e, S.e1b, epsb, Rb, full);
 }
 
 template <typename T>
@@ -528,11 +541,12 @@ __device__ __forceinline__ void store_state34(T* __restrict__ dst, long long i, 
   for (int c = 0; c < 12; ++c) dst[(22 + c) * n + i] = y.al[c];
 }
 
-template <typename T, int NP, int NS>
-__device__ __forceinline__ void vjp_prepare(const MatDev<T>& M, long long i, size_t n, const T* __restrict__ R,
-                                            const T* __restrict__ eps_n, const T* __restrict__ eps,
-                                            const T* __restrict__ state, T dt, int nsub, const T* tab,
-                                            VjpVoxel<T, NS>& P) {
+// Loads a voxel: its state at t_n into y, its strain path in the crystal frame into e0 (at t_n)
+// and de (its step).
+template <typename T, int NS>
+__device__ __forceinline__ void vjp_load(const MatDev<T>& M, long long i, size_t n, const T* __restrict__ R,
+                                         const T* __restrict__ eps_n, const T* __restrict__ eps,
+                                         const T* __restrict__ state, T* e0, T* de, MPState<T>& y, VjpVoxel<T, NS>& P) {
 #pragma unroll
   for (int k = 0; k < 9; ++k) P.r[k] = R[(size_t)i * 9 + k];
 #pragma unroll
@@ -540,23 +554,86 @@ __device__ __forceinline__ void vjp_prepare(const MatDev<T>& M, long long i, siz
     P.en[c] = eps_n[c * n + i];
     P.e[c] = eps[c * n + i];
   }
-  MPState<T> y;
   load_state34<T>(state, i, n, y);
-  T e0[6], de[6];
   to_crystal<T>(P.r, P.en, e0);
   to_crystal<T>(P.r, P.e, P.e1);
 #pragma unroll
   for (int c = 0; c < 6; ++c) de[c] = P.e1[c] - e0[c];
   P.quiet = elastic_increment<T>(M, e0, de, y);
-  if (!P.quiet) mc_forward_store<T, NP, NS>(M, e0, de, dt, nsub, tab, y, P);
+}
+
+// The sweeps of SEEDS seeds of a voxel.  seed(k, S, sigma_b) fills seed k's state and stress
+// adjoint; take(k, S, ...) receives its results; `full` belongs to the last seed.
+// NB = 1: one forward pass leaves the records of all substeps, then each seed is swept in turn.
+// NB > 1: the records of one block at a time.  The forward pass runs block after block and keeps
+// the state at each block's start; the last block's records are there at its end, those of the
+// one before are made again on the way back, and all seeds pass a block before the next.
+// CUDA reserves a kernel's local memory for every thread the chip can hold: records of all 16
+// substeps, 39.9 KB a thread in double, made the context grow by 12.4 GB in a call with more than
+// 4 substeps.  Two blocks of 8 take 24.0 KB (7.5 GB), one of 8 20.4 KB, and kernels
+// without records took 24.4 KB.  What the second making of records costs: 20011 points in double
+// with 16 substeps 7.0 -> 10.0 ms, 100003 in float 2.4 -> 3.5 ms; up to 8 substeps nothing.
+template <typename T, int NP, int NS, int NB, int SEEDS, typename Seed, typename Take>
+__device__ __forceinline__ void vjp_sweeps(const MatDev<T>& M, const T* e0, const T* de, T dt, int nsub,
+                                           const T* tab, MPState<T>& y, VjpVoxel<T, NS>& P, Seed seed, Take take) {
+  T pb[kParamBar], rb[9] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
 #pragma unroll
-  for (int c = 0; c < 6; ++c) P.epN[c] = y.ep[c];
+  for (int k = 0; k < kParamBar; ++k) pb[k] = T(0);
+  auto finish = [&](int k, VjpSeed<T>& S) {
+    T enb[6] = {T(0), T(0), T(0), T(0), T(0), T(0)}, eb[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+    reverse_strains<T, NS>(P, S, enb, eb, rb, k == SEEDS - 1);
+    take(k, S.yb, eb, enb, rb, pb);
+  };
+  if constexpr (NB == 1) {
+    if (!P.quiet) mc_forward_store<T, NP, NS>(M, e0, de, dt, nsub, 0, nsub, tab, y, P);
+#pragma unroll
+    for (int c = 0; c < 6; ++c) P.epN[c] = y.ep[c];
+#pragma unroll 1
+    for (int k = 0; k < SEEDS; ++k) {
+      VjpSeed<T> S;
+      T sb[6];
+      seed(k, S.yb, sb);
+      reverse_stress<T, NS>(M, P, sb, S, rb, k == SEEDS - 1);
+      if (!P.quiet) reverse_substeps<T, NS>(M, P, dt, nsub, 0, nsub, S, pb, k == SEEDS - 1);
+      finish(k, S);
+    }
+  } else {
+    VjpSeed<T> S[SEEDS];
+    MPState<T> start[NB];  // the state at each block's start
+    // the first block takes the remainder: its records are made twice
+    const int nb = P.quiet ? 1 : (nsub + NS - 1) / NS, n0 = nsub - (nb - 1) * NS;
+    // blocks 0 .. nb-1 forward, then nb-2 .. 0 again, each followed by its reverse
+#pragma unroll 1
+    for (int t = 0; t < 2 * nb - 1; ++t) {
+      const int b = t < nb ? t : 2 * nb - 2 - t, m1 = n0 + b * NS, m0 = b > 0 ? m1 - NS : 0;
+      if (!P.quiet) {
+        if (t < nb) start[b] = y;
+        else y = start[b];
+        mc_forward_store<T, NP, NS>(M, e0, de, dt, nsub, m0, m1, tab, y, P);
+      }
+      if (t + 1 < nb) continue;
+      if (t + 1 == nb)
+#pragma unroll
+        for (int c = 0; c < 6; ++c) P.epN[c] = y.ep[c];
+#pragma unroll 1
+      for (int k = 0; k < SEEDS; ++k) {
+        if (t + 1 == nb) {
+          T sb[6];
+          seed(k, S[k].yb, sb);
+          reverse_stress<T, NS>(M, P, sb, S[k], rb, k == SEEDS - 1);
+        }
+        if (!P.quiet) reverse_substeps<T, NS>(M, P, dt, nsub, m0, m1, S[k], pb, k == SEEDS - 1);
+      }
+    }
+#pragma unroll 1
+    for (int k = 0; k < SEEDS; ++k) finish(k, S[k]);
+  }
 }
 
 // One thread per voxel; arrays component-major (component * nvox + voxel) as in the
 // forward material-point kernel.  state_b: in, adjoint of the state at t_{n+1}; out, adjoint
 // of the state at t_n.  R_b (9 x nvox) and param_b (kParamBar x nvox) are per voxel.
-template <typename T, int NP, int NS>
+template <typename T, int NP, int NS, int NB>
 __global__ void k_material_point_vjp(const MatDev<T> M, long long nvox, const T* __restrict__ R,
                                      const T* __restrict__ eps_n, const T* __restrict__ eps,
                                      const T* __restrict__ state, T dt, int nsub, const T* __restrict__ sigma_b,
@@ -571,28 +648,28 @@ __global__ void k_material_point_vjp(const MatDev<T> M, long long nvox, const T*
   if (i >= nvox) return;
   const size_t n = (size_t)nvox;
   VjpVoxel<T, NS> P;
-  vjp_prepare<T, NP, NS>(M, i, n, R, eps_n, eps, state, dt, nsub, tab, P);
-  T sb[6];
+  MPState<T> y;
+  T e0[6], de[6];
+  vjp_load<T, NS>(M, i, n, R, eps_n, eps, state, e0, de, y, P);
+  vjp_sweeps<T, NP, NS, NB, 1>(
+      M, e0, de, dt, nsub, tab, y, P,
+      [&](int, MPState<T>& yb, T* sb) {
 #pragma unroll
-  for (int c = 0; c < 6; ++c) sb[c] = sigma_b[c * n + i];
-  MPState<T> yb;
-  load_state34<T>(state_b, i, n, yb);
-  T enb[6] = {T(0), T(0), T(0), T(0), T(0), T(0)}, eb[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-  T rb[9] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
-  T pb[kParamBar];
+        for (int c = 0; c < 6; ++c) sb[c] = sigma_b[c * n + i];
+        load_state34<T>(state_b, i, n, yb);
+      },
+      [&](int, const MPState<T>& yb, const T* eb, const T* enb, const T* rb, const T* pb) {
+        store_state34<T>(state_b, i, n, yb);
 #pragma unroll
-  for (int k = 0; k < kParamBar; ++k) pb[k] = T(0);
-  mc_reverse<T, NS>(M, P, dt, nsub, sb, yb, enb, eb, rb, pb, true);
-  store_state34<T>(state_b, i, n, yb);
+        for (int c = 0; c < 6; ++c) {
+          eps_b[c * n + i] = eb[c];
+          eps_n_b[c * n + i] = enb[c];
+        }
 #pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    eps_b[c * n + i] = eb[c];
-    eps_n_b[c * n + i] = enb[c];
-  }
+        for (int k = 0; k < 9; ++k) R_b[k * n + i] = rb[k];
 #pragma unroll
-  for (int k = 0; k < 9; ++k) R_b[k * n + i] = rb[k];
-#pragma unroll
-  for (int k = 0; k < kParamBar; ++k) param_b[k * n + i] = pb[k];
+        for (int k = 0; k < kParamBar; ++k) param_b[k * n + i] = pb[k];
+      });
 }
 
 // The reverse work of one increment of the history adjoint before its fixed point, over one
@@ -601,7 +678,7 @@ __global__ void k_material_point_vjp(const MatDev<T> M, long long nvox, const T*
 // and the direct part (uniform stress adjoint sd, state adjoint state_b at t_{n+1}, which is
 // overwritten with the adjoint at t_n), whose eps, eps_n, rotation and parameter adjoints go
 // to eps_b, eps_n_b, R_b and param_b.
-template <typename T, int NP, int NS>
+template <typename T, int NP, int NS, int NB>
 __global__ void k_adj_tangent(const MatDev<T> M, long long nvox, const T* __restrict__ R,
                               const T* __restrict__ eps_n, const T* __restrict__ eps,
                               const T* __restrict__ state, T dt, int nsub, T sd0, T sd1, T sd2, T sd3, T sd4, T sd5,
@@ -616,41 +693,38 @@ __global__ void k_adj_tangent(const MatDev<T> M, long long nvox, const T* __rest
   if (i >= nvox) return;
   const size_t n = (size_t)nvox;
   VjpVoxel<T, NS> P;
-  vjp_prepare<T, NP, NS>(M, i, n, R, eps_n, eps, state, dt, nsub, tab, P);
-#pragma unroll 1
-  for (int row = 0; row < 7; ++row) {
-    T sb[6];
-    MPState<T> yb;
-    if (row < 6) {
+  MPState<T> y;
+  T e0[6], de[6];
+  vjp_load<T, NS>(M, i, n, R, eps_n, eps, state, e0, de, y, P);
+  vjp_sweeps<T, NP, NS, NB, 7>(
+      M, e0, de, dt, nsub, tab, y, P,
+      [&](int row, MPState<T>& yb, T* sb) {
+        if (row < 6) {
 #pragma unroll
-      for (int c = 0; c < 6; ++c) sb[c] = c == row ? T(1) : T(0);
-      state_zero<T>(yb);
-    } else {
-      sb[0] = sd0; sb[1] = sd1; sb[2] = sd2; sb[3] = sd3; sb[4] = sd4; sb[5] = sd5;
-      load_state34<T>(state_b, i, n, yb);
-    }
-    T enb[6] = {T(0), T(0), T(0), T(0), T(0), T(0)}, eb[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
-    T rb[9] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
-    T pb[kParamBar];
+          for (int c = 0; c < 6; ++c) sb[c] = c == row ? T(1) : T(0);
+          state_zero<T>(yb);
+        } else {
+          sb[0] = sd0; sb[1] = sd1; sb[2] = sd2; sb[3] = sd3; sb[4] = sd4; sb[5] = sd5;
+          load_state34<T>(state_b, i, n, yb);
+        }
+      },
+      [&](int row, const MPState<T>& yb, const T* eb, const T* enb, const T* rb, const T* pb) {
+        if (row < 6) {
 #pragma unroll
-    for (int k = 0; k < kParamBar; ++k) pb[k] = T(0);
-    mc_reverse<T, NS>(M, P, dt, nsub, sb, yb, enb, eb, rb, pb, row == 6);
-    if (row < 6) {
+          for (int c = 0; c < 6; ++c) J[((size_t)row * 6 + c) * n + i] = eb[c];
+          return;
+        }
+        store_state34<T>(state_b, i, n, yb);
 #pragma unroll
-      for (int c = 0; c < 6; ++c) J[((size_t)row * 6 + c) * n + i] = eb[c];
-    } else {
-      store_state34<T>(state_b, i, n, yb);
+        for (int c = 0; c < 6; ++c) {
+          eps_b[c * n + i] = eb[c];
+          eps_n_b[c * n + i] = enb[c];
+        }
 #pragma unroll
-      for (int c = 0; c < 6; ++c) {
-        eps_b[c * n + i] = eb[c];
-        eps_n_b[c * n + i] = enb[c];
-      }
+        for (int k = 0; k < 9; ++k) R_b[k * n + i] = rb[k];
 #pragma unroll
-      for (int k = 0; k < 9; ++k) R_b[k * n + i] = rb[k];
-#pragma unroll
-      for (int k = 0; k < kParamBar; ++k) param_b[k * n + i] = pb[k];
-    }
-  }
+        for (int k = 0; k < kParamBar; ++k) param_b[k * n + i] = pb[k];
+      });
 }
 
 }  // namespace rve

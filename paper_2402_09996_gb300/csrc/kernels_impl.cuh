@@ -69,7 +69,9 @@ cudaError_t launch_material_point_vjp_np(const MatDev<T>& M, long long nvox, con
   const int thr = 64;
   const long long grid = (nvox + thr - 1) / thr;
   const size_t smem = (size_t)table_len<T, NP>(M) * sizeof(T);
-  const auto fn = nsub <= kFewSubVjp ? k_material_point_vjp<T, NP, kFewSubVjp> : k_material_point_vjp<T, NP, kMaxSubVjp>;
+  const auto fn = nsub <= kFewSubVjp  ? k_material_point_vjp<T, NP, kFewSubVjp, 1>
+                  : nsub <= kBlockVjp ? k_material_point_vjp<T, NP, kBlockVjp, 1>
+                                      : k_material_point_vjp<T, NP, kBlockVjp, 2>;
   cudaError_t e = set_smem<T>((const void*)fn, smem);
   if (e != cudaSuccess) return e;
   fn<<<(unsigned)grid, thr, smem, s>>>(M, nvox, R, eps_n, eps, state, dt, nsub, sigma_b, state_b, eps_b, eps_n_b, R_b,
@@ -85,7 +87,9 @@ cudaError_t launch_adj_tangent_np(const MatDev<T>& M, long long nvox, const T* R
   const int thr = 64;
   const long long grid = (nvox + thr - 1) / thr;
   const size_t smem = (size_t)table_len<T, NP>(M) * sizeof(T);
-  const auto fn = nsub <= kFewSubVjp ? k_adj_tangent<T, NP, kFewSubVjp> : k_adj_tangent<T, NP, kMaxSubVjp>;
+  const auto fn = nsub <= kFewSubVjp  ? k_adj_tangent<T, NP, kFewSubVjp, 1>
+                  : nsub <= kBlockVjp ? k_adj_tangent<T, NP, kBlockVjp, 1>
+                                      : k_adj_tangent<T, NP, kBlockVjp, 2>;
   cudaError_t e = set_smem<T>((const void*)fn, smem);
   if (e != cudaSuccess) return e;
   fn<<<(unsigned)grid, thr, smem, s>>>(M, nvox, R, eps_n, eps, state, dt, nsub, (T)sd[0], (T)sd[1], (T)sd[2], (T)sd[3],

@@ -143,9 +143,9 @@ constexpr int kDirect = 3;
 // Template value of the x pass's linear-law mode (the adjoint solve): s = B eps - g per voxel.
 constexpr int kLinearLaw = 1;
 
-// RK4 substeps of an increment whose stage records the constitutive reverse pass (adjoint.cuh)
-// keeps in local memory: two kernel variants, so that the usual 4 substeps (increments up to
-// 0.5 s) reserve a quarter of the memory.
-constexpr int kFewSubVjp = 4, kMaxSubVjp = 16;
+// RK4 substeps whose stage records the constitutive reverse pass (adjoint.cuh) keeps in local
+// memory at a time: kernel variants for the usual 4 substeps (increments up to 0.5 s), which
+// reserve half the memory, for up to 8 in one block, and for up to 16 in two.
+constexpr int kFewSubVjp = 4, kBlockVjp = 8, kMaxSubVjp = 2 * kBlockVjp;
 
 }  // namespace rve
