@@ -18,7 +18,7 @@ template <typename T> struct ZGroup;
 struct GuardGroup;
 
 // Rate-solve variants of the constitutive kernels (see constitutive.cuh): kDirect where both
-// laws have a direct table (2 <= n <= 10.2), NP = -1 for other exponents >= 1, and NP = 0
+// laws have a direct table (rate_law_fit: 2 <= n <= 10.2), NP = -1 for other exponents >= 1, and NP = 0
 // (generic per-system solve) for eta = 0.
 template <typename T>
 inline int rate_variant(double eta, double K, double n, double Kt, double nt) {

@@ -15,8 +15,11 @@
 // S and the octaves below K follow from n (rate_law_fit): the table starts where F falls below
 // 2^-100 and takes the finest S that leaves at least 5 octaves above K.  For 2 <= n <= 10.2
 // the relative error against the exact root is then below 2.1e-7 in float and 2.4e-16 in
-// double over the whole table, rounding included; the power law needs finer segments for
-// larger n and more octaves for smaller n (those laws take the Newton variants).
+// double for all F >= 2^-100 in the table, rounding included; the power law needs finer segments
+// for larger n and more octaves for smaller n (those laws take the Newton variants).  The
+// cubic's last coefficient is about n^3/6 F/a^3: in float it is subnormal, and lost, at small
+// rates of a large K (relative errors of 2.8e-7 at K = 1e8, 3e-3 at 1e12, against 2.1e-7 at 3e7),
+// so float tables end at K = 1e7.
 // Below the table the float rate is 0 (< 2^-100 per second); above it the last segment
 // holds NaN, which reaches the voxel's stress, and the voxel is integrated again by the
 // generic solve.  Double solves generically outside the table.
@@ -31,11 +34,13 @@ template <> struct RateFmt<float> {
   static constexpr int kDeg = 3, kSeries = 8, kSegs = 1408, kFine = 6;
   static constexpr int kRow = kDeg + 1;
   static constexpr int kLen = (kSegs + 2) * kRow;  // zero segment, polynomials, NaN segment
+  static constexpr double kKmax = 1e7;
 };
 template <> struct RateFmt<double> {
   static constexpr int kDeg = 9, kSeries = 16, kSegs = 704, kFine = 5;
   static constexpr int kRow = kDeg + 1;
   static constexpr int kLen = kSegs * kRow;
+  static constexpr double kKmax = 1e12;
 };
 
 // 2^(j/64), j = 0 .. 63, follow the law tables in double (exp2_tab)
@@ -50,8 +55,8 @@ struct RateGrid {
 };
 
 // Host: the table grid of a law, or false where no table is built.
-inline bool rate_law_fit(double K, double n, double eta, int segs, int fine, RateGrid* g) {
-  if (!(eta > 0.0) || !(n >= 2.0 && n <= 10.2) || !(K >= 1e-6 && K <= 1e12)) return false;
+inline bool rate_law_fit(double K, double n, double eta, int segs, int fine, double K_max, RateGrid* g) {
+  if (!(eta > 0.0) || !(n >= 2.0 && n <= 10.2) || !(K >= 1e-6 && K <= K_max)) return false;
   int below = 1;
   while (below * n < 100.0) ++below;
   for (int S = fine; S > fine - 3; --S) {
@@ -69,7 +74,7 @@ inline bool rate_law_fit(double K, double n, double eta, int segs, int fine, Rat
 
 template <typename T>
 inline bool rate_law_fit_t(double K, double n, double eta, RateGrid* g) {
-  return rate_law_fit(K, n, eta, RateFmt<T>::kSegs, RateFmt<T>::kFine, g);
+  return rate_law_fit(K, n, eta, RateFmt<T>::kSegs, RateFmt<T>::kFine, RateFmt<T>::kKmax, g);
 }
 
 inline RateLaw<float> rate_law_f(const RateGrid& g, int off) {
