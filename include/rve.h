@@ -80,7 +80,7 @@ typedef struct {
                          handle's stream and accumulate per-kernel times (rve_kernel_times) */
   int graphs;         /* nonzero (default): run each increment's fixed-point loop on the device
                          as one CUDA graph launch (a conditional while-node repeats the
-                         iteration until the residual kernel decides; the commit follows in the
+                         iteration until the device decides; the commit follows in the
                          same graph), so the host waits once per increment.  The graphs are
                          built on first use per buffer rotation (three per handle) and rebuilt
                          after rve_set_mixed_load changes the load.  Ignored when timing is set. */

@@ -237,7 +237,7 @@ struct rve_s {
   unsigned char* flow = nullptr;  // x pass: per warp of 32 voxels, flowed in iteration 0 (XArgs::flow)
   uint32_t* grain = nullptr;
   void* Rg = nullptr;
-  void* root_tab = nullptr;  // kRootTabs rate-root table values (slip systems, twin exponent)
+  void* root_tab = nullptr;  // the material's rate tables: tables_of values (room: root_tab_bytes)
   void *tw_x = nullptr, *tw_y = nullptr, *tw_z = nullptr;
   void *kx = nullptr, *ky = nullptr, *kz = nullptr;
   double* partial = nullptr;
@@ -575,7 +575,11 @@ size_t z_smem(const rve_s* h, int hc) {
 // rounds).  The pass is bound by the constitutive update, so the busiest SM's rounds,
 // ceil(CTAs / 152) r, set its time; among equals, the fewest rounds in sequence, counting half
 // a round per CTA for its transforms and table copy (`resident` CTAs share an SM), then the
-// larger L.  At most 5 rounds, which keeps 3 float CTAs per SM in shared memory.  Measured x
+// larger L.  At most 5 rounds, which keeps 3 float CTAs per SM in shared memory with the tables of
+// one law (two laws: 2 at 5 rounds; in double 2 with one law up to 4 rounds, else 1).  `resident` is the
+// count by registers all the same: with the count by shared memory, the rule chose wider CTAs
+// for two laws in double, x pass 32^3 816 (L = 4) -> 920 us (8), 40^3 1672 (6) -> 1736 (12),
+// 60^3 5089 (6) -> 5024 (8), and the same L for float cubes up to 256.  Measured x
 // passes: 48^3 FP64 L = 8 2.06 ms (7: 2.78, 5: 2.53, 16: 2.50), 32^3 FP64 L = 4 0.72 (8: 0.86),
 // 20^3 FP64 L = 6 0.41 (7: 0.70), 64^3 FP32 L = 4 141 us (8: 156, 2: 150), 96^3 L = 4 383
 // (5: 401), 128^3 L = 4 804 (3: 824, 5: 815, 2: 863), 160^3 L = 4 1536 (3: 1598, 5: 1596).
@@ -974,7 +978,7 @@ rve_status enqueue_one(rve_s* h, cudaStream_t s, int it, int si, int so, int pi,
 }
 
 // Enqueues iterations inc_it0 .. inc_it0 + inc_nb - 1, then the status copy and ev_sync.
-// The residual kernel decides convergence on the device; later launches of the batch
+// The inverse y pass decides convergence on the device (resid_update); later launches of the batch
 // return at once.
 template <typename T>
 rve_status enqueue_iterations(rve_s* h) {
@@ -997,7 +1001,7 @@ bool use_graphs(const rve_s* h) { return h->opt.graphs && !h->opt.timing; }
 // (S0 -> S1), then a while-node whose body runs two iterations (S1 -> S2, S2 -> S1) and a
 // guard kernel, then the commit (a no-op unless the increment converged; it reads the
 // converged iteration's spectrum) and the status copy to the host.  The loop ends when the
-// residual kernel decides (converged, NaN, or the iteration cap) or, independently, after
+// inverse y pass decides (converged, NaN, or the iteration cap) or, independently, after
 // max_iter / 2 + 2 body executions.
 template <typename T>
 rve_status build_graph(rve_s* h) {

@@ -458,8 +458,8 @@ __device__ __forceinline__ void xpass_cta(const XArgs<T>& a, const XCommon<T>& k
   double acc[kNumRed];
 #pragma unroll
   for (int i = 0; i < kNumRed; ++i) acc[i] = 0.0;
-  // the thread's stresses are summed in the field precision over its few voxels (4 at
-  // most in float) and added to the FP64 block sum once
+  // the thread's stresses are summed in the field precision over its few voxels (5 at
+  // most) and added to the FP64 block sum once
   T sacc[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
   bool quad = false;
   if constexpr (std::is_same<T, double>::value && NP == kDirect) {
@@ -1156,7 +1156,7 @@ __global__ void __launch_bounds__(N1 > 0 ? kPencilThreads : kZThreads, ZMinBlock
 }
 
 // Graph mode: second bound on the device-side iteration loop, independent of the
-// residual kernel's decision: after `limit` executions of the loop body (two iterations
+// residual's decision: after `limit` executions of the loop body (two iterations
 // each) the loop condition is cleared.
 template <typename T>
 __global__ void k_loop_guard(IterStatus* st, int limit, cudaGraphConditionalHandle cond) {
