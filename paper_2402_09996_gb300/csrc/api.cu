@@ -1090,6 +1090,7 @@ rve_status tune_tiles(rve_s* h) {
   RVE_CUDA(h, cudaMemsetAsync(sp, 0, spec_bytes, s));
   RVE_CUDA(h, cudaMemsetAsync(pp, 0, spec_bytes, s));
   RVE_CUDA(h, cudaMemsetAsync(h->st_tune, 0, sizeof(IterStatus), s));
+  RVE_CUDA(h, cudaMemsetAsync(h->partial, 0, (size_t)h->xgrid * 6 * sizeof(double), s));
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   RVE_CUDA(h, cudaEventCreate(&e0));
   cudaError_t e = cudaEventCreate(&e1);
@@ -1119,10 +1120,12 @@ rve_status tune_tiles(rve_s* h) {
       prev = hc;
       const size_t sm = y_smem<T>(h, hc);
       if (sm > (size_t)smax) continue;
-      LineArgs<T> ya = y_args<T>(h, sp);
+      // the forward pass as an iteration launches it, its side work on the scratch status
+      LineArgs<T> ya = y_pass_args<T>(h, sp, kSideMean, 0);
       ya.HC = hc;
-      ya.done = nullptr;
-      const dim3 grid((h->H + hc - 1) / hc, h->nz);
+      ya.side.st = h->st_tune;
+      ya.done = &h->st_tune->done;
+      const dim3 grid((h->H + hc - 1) / hc, h->nz + 1);
       float ms = 0.f;
       e = timed([&] { return launch_line<T>(ya, -1, grid, sm, s); }, &ms);
       if (e != cudaSuccess) break;

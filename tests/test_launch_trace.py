@@ -39,3 +39,14 @@ def test_material_tables_are_complete_when_the_call_returns(trace):
     not wait for work that rve_set_material leaves in flight."""
     calls = trace("material")
     assert "rate_table" in calls and calls[-1] == "sync"
+
+
+def test_autotuner_times_the_pass_that_runs(trace):
+    """The widths of the y tile are timed on the forward pass with its side work (an extra row
+    of CTAs), which is what an iteration launches."""
+    lines = [re.search(r"sign=(-?\d) kind=(\d) goes_by=(\w+) HC=(\d+) grid=\d+,(\d+) nz=(\d+)", t).groups()
+             for t in trace("tune") if t.startswith("line")]
+    first = next(k for k, t in enumerate(lines) if t[0] == "1")  # the first inverse pass
+    tuned = lines[: first - 1]
+    assert len({t[3] for t in tuned}) == 5
+    assert all(t[1] == "1" and int(t[4]) == int(t[5]) + 1 for t in tuned)
