@@ -56,9 +56,14 @@ ENSEMBLE_WORKLOAD = ("ensemble of 16 RVEs: 4 each of 64^3, 96^3, 128^3, 160^3 vo
 WORKLOAD_128 = ("twinned RVE 128^3, 200 Voronoi grains (p_twin 0.5), FP32 fields + FP64 norms, uniaxial tension "
                 "1e-3/s, dt 0.5 s")
 # algorithmic work per voxel-iteration: state in + stress out + one spectral round trip (bytes);
-# four RK stages per substep, each one right-hand side with its rate-root solves (flops)
+# four RK stages per substep, each one right-hand side (flops; an FMA is two, an exponential or
+# logarithm one, comparisons and sign changes none)
 BYTES_PER_VOXIT_FP32 = 260          # state + strain/stress traffic of the fused iteration
-FLOPS_RHS = 1100                    # one evaluation of the constitutive right-hand side
+# One evaluation of the constitutive right-hand side by the float stage with direct rate tables
+# (rk_stage): strain and stress 35, hardening terms and their sums 55, prefactors and resistances
+# 18, plane sums 12, slip systems 12 x 24 (of which the rate 7) + 30 for their sums, twins
+# 4 x 20 + 12, plastic strain 46.
+FLOPS_RHS = 35 + 55 + 18 + 12 + 12 * 24 + 30 + 4 * 20 + 12 + 46
 N_SUB = 4                           # RK4 substeps at dt = 0.5 s
 DT = 0.5
 # DRAM bytes (read + write) of one trial x-pass launch on the twinned 128^3 FP32 case, from
