@@ -612,9 +612,10 @@ __device__ __forceinline__ void vjp_sweeps(const MatDev<T>& M, const T* e0, cons
         mc_forward_store<T, NP, NS>(M, e0, de, dt, nsub, m0, m1, tab, y, P);
       }
       if (t + 1 < nb) continue;
-      if (t + 1 == nb)
+      if (t + 1 == nb) {
 #pragma unroll
         for (int c = 0; c < 6; ++c) P.epN[c] = y.ep[c];
+      }
 #pragma unroll 1
       for (int k = 0; k < SEEDS; ++k) {
         if (t + 1 == nb) {
